@@ -91,6 +91,11 @@ struct ItemDesc {
   // exact path constants
   float c1f, c2f, c1cf, c3f, S0f, Kf;
   double c1d, c2d, c1cd, c3d, S0d, Kd;
+  // FP64 exact path, increments in units 2^-qF (0: they may reach 8, the kernel
+  // forms them in FP64): q1 = c1 - c3 (c1 for Euler), q2 = c2 2^4, q3 = c3 2^8
+  int64_t q1;
+  uint64_t q2, q3;
+  int32_t qF, q_pad;
   // approximate path
   FixedConsts fx;
   FastFixed ff;

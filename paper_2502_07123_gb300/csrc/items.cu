@@ -426,6 +426,26 @@ bool sample_range_ok(int level, uint64_t first, uint64_t N) {
   return N <= (1ULL << 58) && N <= words && first <= words - N;
 }
 
+// Integer increments of the FP64 exact path (exact64.cuh): the unit 2^-qF keeps
+// |increment| < 2^61 units for every |Z| < 6.4 (Phi^-1(2^-33) = -6.34; the coarse
+// step adds two).  With y = |Z| 2^60 the products' factors then satisfy
+// mulhi64_3's bound: high words of q2 and y below 2^33 / 6.4 + 6.34 2^28, of y
+// and y' below 6.34 2^29, of q3 and y y' 2^-64 below 2^37 / 43 + 40.2 2^24.
+// Increments that may reach 8 (sigma sqrt(h) above about 0.6) stay in FP64.
+void exact64_consts(ItemDesc &it, bool milstein) {
+  const double zmax = 6.4, c3 = milstein ? it.c3d : 0.0;
+  const double z = it.level > 0 ? 2.0 * zmax : zmax;
+  const double b = std::fabs(it.level > 0 ? it.c1cd : it.c1d) + it.c2d * z + c3 * (z * z + 2.0);
+  it.qF = 0;
+  if (!(b < 8.0)) return;
+  const int k = b > 0x1p-8 ? std::ilogb(b) + 1 : -7;   // b < 2^k
+  it.qF = 61 - k;
+  // (Milstein: plus the mean of what the truncated products of c3 Z^2 lose)
+  it.q1 = std::llround(std::ldexp(it.c1d, it.qF)) - std::llround(std::ldexp(c3, it.qF)) + (milstein ? 1 : 0);
+  it.q2 = (uint64_t)std::ldexp(it.c2d, it.qF + 4);
+  it.q3 = (uint64_t)std::ldexp(c3, it.qF + 8);
+}
+
 mlmc_status build_item(const mlmc_work &w, int out_index, void *dump, BuiltItem &b, double &disc, int &unit,
                        int &exact_int, TableSource &src) {
   const mlmc_params *p = w.params;
@@ -487,6 +507,7 @@ mlmc_status build_item(const mlmc_work &w, int out_index, void *dump, BuiltItem 
   it.c1d = rh; it.c2d = c2; it.c1cd = rh2; it.c3d = c3; it.S0d = p->S0; it.Kd = p->K;
   it.c1f = (float)rh; it.c2f = (float)c2; it.c1cf = (float)rh2; it.c3f = (float)c3;
   it.S0f = (float)p->S0; it.Kf = (float)p->K;
+  if (v == MLMC_FP64_EXACT) exact64_consts(it, p->scheme == MLMC_MILSTEIN);
   disc = std::exp(-p->r * p->T);
   unit = 0;
   exact_int = 0;

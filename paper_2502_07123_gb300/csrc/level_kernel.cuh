@@ -15,6 +15,7 @@
 #include <type_traits>
 
 #include "device_common.cuh"
+#include "exact64.cuh"
 #include "mlmc.h"
 #include "reduce.cuh"
 
@@ -72,10 +73,12 @@ __device__ __forceinline__ void stage_phi_inv() {
   float4 *d = phi_inv_smem();
   for (int k = threadIdx.x; k < PHI_INV_PARTS; k += blockDim.x) d[k] = k_phi_inv[k];
 }
+// The exact path's inverse-Normal table of a kernel, if it has one.
 template <int EST, int XP>
-struct NeedsPhi {
-  static constexpr bool value = EST != EST_APPROX && XP == XP_F32;
-};
+__device__ __forceinline__ void stage_exact_table() {
+  if constexpr (EST != EST_APPROX && XP == XP_F32) stage_phi_inv();
+  if constexpr (EST != EST_APPROX && XP == XP_F64) stage_phi64();
+}
 
 // Bytes per entry of the shared-memory approximate-Normal table of a datapath:
 // the 32-bit fast fixed-point datapath keeps (Z~_j, sum1 of a fine step) pairs.
@@ -114,7 +117,8 @@ __device__ __forceinline__ int32_t ff_sum1(const FastFixed &ff, int32_t z, int32
 // MSEL: 0 the item uses a table lookup (Methods 1 and 2), 1 the line
 // evaluation of Method 3, 2 either, chosen per step (only the per-sample
 // dump instantiation); chosen once per chunk, so the hot step code has no
-// branch on the method.
+// branch on the method.  FP64 exact kernels: 0 increments in 64-bit integers
+// (exact64.cuh), 1 in FP64.
 // PRE (merged nested kernel, family 24): the 32-bit fast datapath's sum1
 // arrives multiplied by 2^(32 - rs2) (the host proved that it fits), so the
 // rounded product rd(S sum1) is the high word of one 64-bit multiply-add: no
@@ -167,6 +171,12 @@ struct LevelSim {
   const float4 *phi;       // FP32 exact path: the inverse-Normal cubics in shared memory
   uint32_t low_mask;
   X c1, c2, c1c, c3, S0, K;
+  // FP64 exact path: integer increments (exact64.cuh)
+  int64_t q1;
+  uint64_t q2, q3;
+  int qF;
+  uint32_t qhi;            // q_to_double's exponent word
+  const ulonglong2 *phi64;
   // fixed point
   FixedConsts fx;
   FastFixed ff;
@@ -180,6 +190,9 @@ struct LevelSim {
 
   // ---- per-sample state (approximate state per lane) ----
   X S, Sc, zprev, accF, accC, minF, minC;
+  int64_t qprev;           // FP64 exact path: the even step's increment, -Phi^-1 and its sign mask
+  uint64_t yprev;
+  int32_t mprev;
   AS aS[KP], aSc[KP], aminF[KP], aminC[KP];
   SatT satb[KP];
   AS hi;   // LAZY: running maximum of S over a group's lanes and steps (reset by the caller)
@@ -199,7 +212,9 @@ struct LevelSim {
     dshift = 32 - it.d;
     method = it.method;
     if constexpr (XP == XP_F64) {
-      c1 = it.c1d; c2 = it.c2d; c1c = it.c1cd; c3 = it.c3d; S0 = it.S0d; K = it.Kd;
+      c1 = it.c1d; c2 = it.c2d; c1c = it.c1cd; c3 = it.c3d; S0 = it.S0d; K = it.Kd + 0.0;   // +0 for a strike of -0 (above_f64)
+      q1 = it.q1; q2 = it.q2; q3 = it.q3; qF = it.qF; qhi = (uint32_t)(1085 - it.qF) << 20;
+      phi64 = phi64_smem();
     } else {
       c1 = it.c1f; c2 = it.c2f; c1c = it.c1cf; c3 = it.c3f; S0 = it.S0f; K = it.Kf;
     }
@@ -262,6 +277,14 @@ struct LevelSim {
   __device__ __forceinline__ bool over() const { return hi > (AS)ff.limT; }
 
   // ---- exact path (FP32 / FP64) ----
+  static __device__ __forceinline__ X lower(X a, X b) {
+    if constexpr (XP == XP_F64) return min_f64(b, a);
+    else return fmin(a, b);
+  }
+  static __device__ __forceinline__ bool above(X a, X b) {   // a > b, b >= 0
+    if constexpr (XP == XP_F64) return above_f64(a, b);
+    else return a > b;
+  }
   __device__ __forceinline__ X exact_inc(X z, X cc1, X mm) const {
     if constexpr (MIL) return fma(c3, fma(z, z, -mm), fma(c2, z, cc1));
     else return fma(c2, z, cc1);
@@ -411,18 +434,52 @@ struct LevelSim {
       // Method 2 (Sec. 3.2): the exact path takes the uniform in the interval
       // pi(j) that the approximate value of j is ranked at, with J's low bits
       const uint32_t Je = perm_s ? (((uint32_t)perm_s[J >> dshift] << dshift) | (J & low_mask)) : J;
-      X z;
-      if constexpr (XP == XP_F64) z = exact_normal_f64(Je);
-      else z = exact_normal_f32(Je, phi);
+      X z, inc;
+      int64_t qi = 0;
+      uint64_t y = 0;
+      int32_t m = 0;
+      const bool qinc = XP == XP_F64 && (MSEL == 2 ? qF != 0 : MSEL == 0);
+      if constexpr (XP == XP_F64) {
+        m = (int32_t)Je >> 31;   // Z = y in the upper half, -y below
+        y = probit_q60(Je ^ (uint32_t)m, phi64);
+        if (qinc) {
+          // c2 Z = +-c2 y, the negative as the complement (one unit 2^-qF off)
+          qi = q1 + (int64_t)(mulhi64_3(q2, y) ^ (uint64_t)(int64_t)~m);
+          if constexpr (MIL) qi += (int64_t)mulhi64_3(q3, mulhi64_3(y, y));
+          inc = q_to_double(qi, qhi);
+        } else {
+          z = q_to_double((int64_t)(y ^ (uint64_t)(int64_t)~m), (uint32_t)(1085 - 60) << 20);
+          inc = exact_inc(z, c1, X(1));
+        }
+      } else {
+        z = exact_normal_f32(Je, phi);
+        inc = exact_inc(z, c1, X(1));
+      }
       if constexpr (PC == PC_ASIAN) { if (i > 0) accF = accF + S; }
-      S = fma(S, exact_inc(z, c1, X(1)), S);
-      if constexpr (PC == PC_LOOKBACK) minF = fmin(minF, S);
+      S = fma(S, inc, S);
+      if constexpr (PC == PC_LOOKBACK) minF = lower(minF, S);
       if constexpr (COARSE) {
         if (odd) {
-          const X zc = zprev + z;
           if constexpr (PC == PC_ASIAN) { if (i > 1) accC = accC + Sc; }
-          Sc = fma(Sc, exact_inc(zc, c1c, X(2)), Sc);
-          if constexpr (PC == PC_LOOKBACK) minC = fmin(minC, Sc);
+          if (qinc) {
+            // c1_c = 2 c1 and (Z + Z')^2 - 2 = (Z^2 - 1) + (Z'^2 - 1) + 2 Z Z': the coarse
+            // increment is the sum of the two fine ones (Milstein: + 2 c3 Z Z')
+            int64_t qc = qprev + qi;
+            if constexpr (MIL) {
+              const uint64_t x = mulhi64_3(q3, mulhi64_3(yprev, y)) << 1;
+              const uint64_t sg = (uint64_t)(int64_t)(mprev ^ m);
+              qc += (int64_t)(x ^ sg);
+            }
+            inc = q_to_double(qc, qhi);
+          } else {
+            inc = exact_inc(zprev + z, c1c, X(2));
+          }
+          Sc = fma(Sc, inc, Sc);
+          if constexpr (PC == PC_LOOKBACK) minC = lower(minC, Sc);
+        } else if (qinc) {
+          qprev = qi;
+          yprev = y;
+          mprev = m;
         } else {
           zprev = z;
         }
@@ -528,19 +585,25 @@ struct LevelSim {
   }
 
   // ---- payoffs ----
-  __device__ __forceinline__ X exact_payoff(X x, X acc, X mn, int steps) const {
+  // lg: log2 of the path's steps
+  __device__ __forceinline__ X exact_payoff(X x, X acc, X mn, int lg) const {
     if constexpr (PC == PC_TERMINAL) {
-      if (payoff == 1) return x > K ? X(1) : X(0);
+      if (payoff == 1) return above(x, K) ? X(1) : X(0);
       const X dd = x - K;
-      return dd > X(0) ? dd : X(0);
+      return above(dd, X(0)) ? dd : X(0);
     } else if constexpr (PC == PC_ASIAN) {
       // one explicit multiply-add: every instantiation rounds the average alike
-      const X avg = fma(X(0.5), x, acc) * (X(1) / X(steps));
+      const X avg = fma(X(0.5), x, acc) * pow2_neg(lg);
       const X dd = avg - K;
-      return dd > X(0) ? dd : X(0);
+      return above(dd, X(0)) ? dd : X(0);
     } else {
       return x - mn;
     }
+  }
+  // 2^-lg (an FP64 division would cost more than the payoff)
+  static __device__ __forceinline__ X pow2_neg(int lg) {
+    if constexpr (XP == XP_F64) return __hiloint2double((1023 - lg) << 20, 0);
+    else return __int_as_float((127 - lg) << 23);
   }
   // PAY: the terminal payoff when known at compile time (0 European, 1 digital), -1 otherwise
   template <int PAY = -1>
@@ -594,8 +657,8 @@ struct LevelSim {
     uint32_t lsat = 0;
     const bool coarse = LV >= 0 ? LV == 1 : level > 0;
     if constexpr (HAS_EXACT) {
-      pf = exact_payoff(S, accF, minF, nsteps);
-      if (coarse) pc = exact_payoff(Sc, accC, minC, nsteps >> 1);
+      pf = exact_payoff(S, accF, minF, level);
+      if (coarse) pc = exact_payoff(Sc, accC, minC, level - 1);
     }
     if constexpr (FIXED) {
       qf = fixed_payoff<PAY>(aS[l], aaccF[l], aminF[l], nsteps, false);
@@ -1206,6 +1269,9 @@ __device__ __forceinline__ void run_chunk(const LaunchArgs &args, const ItemDesc
   const ItemDesc &it = items[item];
   if (ALLOW_DUMP && it.dump) {
     if constexpr (ALLOW_DUMP) chunk_body<EST, XP, AP, SCHEME, PC, KP, 2, true, DYN>(args, it, item, gc, smem_tab);
+  } else if constexpr (XP == XP_F64) {
+    if (it.qF) chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
+    else chunk_body<EST, XP, AP, SCHEME, PC, KP, 1, false, DYN>(args, it, item, gc, smem_tab);
   } else if constexpr (AP == AP_NONE || AP == AP_FX32) {
     // no method choice: exact paths, and the FX32 table that holds every method's values
     chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
@@ -1219,7 +1285,7 @@ __device__ __forceinline__ void run_chunk(const LaunchArgs &args, const ItemDesc
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
 __global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, AP, SCHEME, PC>::value)
 level_kernel(const __grid_constant__ LaunchArgs args) {
-  if constexpr (NeedsPhi<EST, XP>::value) stage_phi_inv();
+  stage_exact_table<EST, XP>();
   run_chunk<EST, XP, AP, SCHEME, PC, KP, false, false>(args, args.items, args.n_items, args.chunk0 + blockIdx.x,
                                                       nullptr);
 }
@@ -1230,7 +1296,7 @@ level_kernel(const __grid_constant__ LaunchArgs args) {
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
 __global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, AP, SCHEME, PC>::value)
 level_kernel_dump(const __grid_constant__ LaunchArgs args) {
-  if constexpr (NeedsPhi<EST, XP>::value) stage_phi_inv();
+  stage_exact_table<EST, XP>();
   run_chunk<EST, XP, AP, SCHEME, PC, KP, true, false>(args, args.items, args.n_items, args.chunk0 + blockIdx.x,
                                                      nullptr);
 }
@@ -1243,7 +1309,7 @@ __global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, AP, SCHEME, PC, t
 level_kernel_dyn(const __grid_constant__ LaunchArgs args) {
   const DynLaunch d = *args.dyn;
   const void *staged = nullptr;
-  if constexpr (NeedsPhi<EST, XP>::value) stage_phi_inv();
+  stage_exact_table<EST, XP>();
   for (uint32_t rel = blockIdx.x; rel < d.n_chunks; rel += gridDim.x)
     run_chunk<EST, XP, AP, SCHEME, PC, KP, false, true>(args, args.items + d.item_off, (int)d.n_items,
                                                         d.chunk0 + rel, &staged);
