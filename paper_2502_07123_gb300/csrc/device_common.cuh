@@ -19,9 +19,10 @@ constexpr uint32_t PHILOX_M1 = 0xCD9E8D57u;
 constexpr uint32_t PHILOX_W0 = 0x9E3779B9u;
 constexpr uint32_t PHILOX_W1 = 0xBB67AE85u;
 
-__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const RoundKeys &rk) {
+__device__ __forceinline__ uint4 philox_rounds(uint4 c, const RoundKeys &rk, int first) {
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
+    if (r < first) continue;
     const uint64_t p0 = (uint64_t)PHILOX_M0 * c.x;
     const uint64_t p1 = (uint64_t)PHILOX_M1 * c.z;
     c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ rk.k[2 * r], (uint32_t)p1,
@@ -29,27 +30,79 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, const RoundKeys &rk) {
   }
   return c;
 }
+__device__ __forceinline__ uint4 philox4x32_10(uint4 c, const RoundKeys &rk) { return philox_rounds(c, rk, 0); }
+
+// Philox calls that differ in the counter's low word only: of the first two
+// rounds' four products two are the same for all of them, as are the words
+// they meet.
+struct PhiloxStream {
+  uint32_t z0, x1, z1, w1;
+  __device__ __forceinline__ PhiloxStream(uint32_t q_hi, uint32_t ctr2, uint32_t ctr3, const RoundKeys &rk) {
+    const uint64_t p = (uint64_t)PHILOX_M1 * ctr2;
+    z0 = ctr3 ^ rk.k[1];
+    x1 = (uint32_t)p ^ rk.k[2];
+    const uint64_t q = (uint64_t)PHILOX_M0 * ((uint32_t)(p >> 32) ^ q_hi ^ rk.k[0]);
+    z1 = (uint32_t)(q >> 32) ^ rk.k[3];
+    w1 = (uint32_t)q;
+  }
+  __device__ __forceinline__ uint4 call(uint32_t q_lo, const RoundKeys &rk) const {
+    const uint64_t p0 = (uint64_t)PHILOX_M0 * q_lo;
+    const uint64_t p1 = (uint64_t)PHILOX_M1 * ((uint32_t)(p0 >> 32) ^ z0);
+    return philox_rounds(make_uint4((uint32_t)(p1 >> 32) ^ x1, (uint32_t)p1, (uint32_t)p0 ^ z1, w1), rk, 2);
+  }
+};
 
 __device__ __forceinline__ uint32_t word_of(const uint4 &w, int k) {
   return k == 0 ? w.x : k == 1 ? w.y : k == 2 ? w.z : w.w;
 }
 
+// 16 bytes from global to shared memory without waiting; the thread waits for
+// all of its copies (copies_done) before the barrier that publishes them.
+__device__ __forceinline__ void copy16_async(void *smem, const void *global) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(smem)), "l"(global)
+               : "memory");
+}
+__device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The inverse-Normal cubics (phi_inv_table.h) in shared memory.  A warp's 32
+// random 16-byte reads of one copy cost 10.4 wavefronts on average (the fullest
+// of 8 bank groups, per quarter warp); beside the pair table's 6.2 they held
+// shared memory 76% busy in the correction kernels.  So the parts of the six octaves [2^-7, 1/2) -- 63 of 64
+// draws -- are kept eight times, one copy per bank group, and lane l reads copy
+// l mod 8: 4 wavefronts and about half a conflict with a rarer part, which is
+// kept once.  19 KB.  8,000,009 level-4 corrections: 317 -> 297 us.
+constexpr int PHI_K0 = 94 << 4;   // exponent field and top four bits of the first part, u = 2^-33
+constexpr int PHI_HOT0 = 26 * 16, PHI_COPIES = 8;
+constexpr int PHI_SMEM = PHI_HOT0 + (PHI_INV_PARTS - PHI_HOT0) * PHI_COPIES;   // in float4
+__device__ __forceinline__ void stage_phi_inv(float4 *d) {
+  for (int k = threadIdx.x; k < PHI_HOT0; k += blockDim.x) copy16_async(d + k, k_phi_inv + k);
+  for (int k = threadIdx.x; k < PHI_SMEM - PHI_HOT0; k += blockDim.x)
+    copy16_async(d + PHI_HOT0 + k, k_phi_inv + PHI_HOT0 + k / PHI_COPIES);
+}
+// What exact_normal_f32 adds to 8 x (exponent and top bits) for the calling lane's copy.
+__device__ __forceinline__ uint32_t phi_lane() {
+  return (threadIdx.x & (PHI_COPIES - 1)) + (uint32_t)(PHI_K0 + PHI_HOT0 - PHI_COPIES * (PHI_K0 + PHI_HOT0));
+}
+
 // Exact Normal Z = Phi^{-1}(2^-32 (J + 1/2)) in single precision (Sec. 3.1).
 // The upper half uses Phi^{-1}(1 - u) = -Phi^{-1}(u): with J' = J or ~J below
 // 2^31, u = 2^-32 (J' + 1/2) (J' rounded to nearest as a float) lies in
-// [2^-33, 1/2].  Phi^{-1}(u) is the cubic of u's part (phi_inv_table.h; tab:
-// that table in shared memory): u's exponent and the top four bits of its
-// significand pick one of 512 parts of [2^-33, 1/2) (the 513th is u = 1/2),
-// the other 19 bits are the position t in [0, 1) within it.  Error: about
-// 1e-7 (1 + |Z|), unbiased (round to nearest).
-__device__ __forceinline__ float exact_normal_f32(uint32_t J, const float4 *tab) {
+// [2^-33, 1/2].  Phi^{-1}(u) is the cubic of u's part (tab: staged as above,
+// lane: phi_lane()): u's exponent and the top four bits of its significand
+// pick one of 512 parts of [2^-33, 1/2) (the 513th is u = 1/2), the other 19
+// bits are the position t in [0, 1) within it, which as the low bits of a
+// float of [16, 17) need no shift.  Error: about 1e-7 (1 + |Z|), unbiased
+// (round to nearest).
+__device__ __forceinline__ float exact_normal_f32(uint32_t J, const float4 *tab, uint32_t lane) {
   const uint32_t m = (uint32_t)((int32_t)J >> 31);
   const float u = fmaf(__uint2float_rn(J ^ m), 0x1p-32f, 0x1p-33f);
   const uint32_t b = __float_as_uint(u);
-  const float4 c = tab[(b >> 19) - (94u << 4)];   // exponent field of 2^-33 is 94
-  const float t = __uint_as_float(((b << 4) & 0x7FFFF0u) | 0x3F800000u) - 1.0f;
+  uint32_t k = b >> 19;
+  if (b >= (uint32_t)(PHI_K0 + PHI_HOT0) << 19) k = k * PHI_COPIES + lane;
+  const float4 c = tab[(int)k - PHI_K0];
+  const float t = __uint_as_float((b & 0x7FFFFu) | 0x41800000u) - 16.0f;
   const float z = fmaf(fmaf(fmaf(c.w, t, c.z), t, c.y), t, c.x);
-  return __int_as_float(__float_as_int(z) ^ (int)(m & 0x80000000u));
+  return __uint_as_float(__float_as_uint(z) ^ (J & 0x80000000u));
 }
 
 __device__ __forceinline__ double exact_normal_f64(uint32_t J) {

@@ -15,6 +15,7 @@
 #pragma once
 #include <stdint.h>
 
+#include "device_common.cuh"
 #include "phi_inv64_table.h"
 
 namespace mlmc {
@@ -30,8 +31,8 @@ __device__ __forceinline__ ulonglong2 *phi64_smem() {
 __device__ __forceinline__ void stage_phi64() {
   ulonglong2 *d = phi64_smem();
   for (int k = threadIdx.x; k < PHI64_HOT; k += blockDim.x) {
-    d[k] = k_phi64_a[k];
-    d[PHI64_HOT + k] = k_phi64_b[k];
+    copy16_async(d + k, k_phi64_a + k);
+    copy16_async(d + PHI64_HOT + k, k_phi64_b + k);
   }
 }
 

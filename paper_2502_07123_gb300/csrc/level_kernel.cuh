@@ -51,32 +51,32 @@ constexpr int MAX_THREADS = 256;
 // kernels of a work list its CTAs fit next to theirs and the step is 3% faster
 // (its device-scheduled form would spill there and keeps its allocation).
 // The approximate 32-bit fixed-point Asian kernels run 4 CTAs per SM (<= 128
-// registers, measured 8-16% faster than their natural ~144).
+// registers, measured 8-16% faster than their natural ~144), as do the
+// corrections whose natural allocation lies just above.
+// The static FP32 exact kernels need 80-87 registers and are held to 80.
 // Every other instantiation keeps its natural allocation (a cap there spills).
 constexpr int LAUNCH_THREADS = 128;
-template <int EST, int AP, int SCHEME, int PC, bool DYN = false> struct MinCtas {
+template <int EST, int XP, int AP, int SCHEME, int PC, bool DYN = false> struct MinCtas {
   static constexpr bool EM_TERMINAL_FX32 = AP == AP_FX32 && SCHEME == 0 && PC == PC_TERMINAL;
   static constexpr int value =
-      (EM_TERMINAL_FX32 && (EST == EST_APPROX || (EST == EST_CORR && !DYN))) ? 6
-      : ((EST == EST_APPROX && AP == AP_FX32 && PC == PC_ASIAN) ? 4 : 1);
+      (EM_TERMINAL_FX32 && (EST == EST_APPROX || (EST == EST_CORR && !DYN))) || (EST == EST_EXACT && XP == XP_F32 && !DYN)
+          ? 6
+      : ((EST == EST_CORR && (AP == AP_FX32 || AP == AP_FX64)) || (EST == EST_APPROX && AP == AP_FX32 && PC == PC_ASIAN)
+             ? 4 : 1);
 };
 
-// The inverse-Normal cubics of the FP32 exact path (phi_inv_table.h) in
-// shared memory: 8 KB, the same for every item.  Kernels whose chunks run an
-// FP32 exact path stage them once per CTA, before their first chunk's table
-// (whose barrier makes them visible).
+// The inverse-Normal cubics of the FP32 exact path in shared memory, the same
+// for every item.  Kernels whose chunks run an FP32 exact path stage them once
+// per CTA, before their first chunk's table (whose barrier makes them visible).
 __device__ __forceinline__ float4 *phi_inv_smem() {
-  __shared__ float4 s_phi_inv[PHI_INV_PARTS];
+  __shared__ float4 s_phi_inv[PHI_SMEM];
   return s_phi_inv;
 }
-__device__ __forceinline__ void stage_phi_inv() {
-  float4 *d = phi_inv_smem();
-  for (int k = threadIdx.x; k < PHI_INV_PARTS; k += blockDim.x) d[k] = k_phi_inv[k];
-}
+
 // The exact path's inverse-Normal table of a kernel, if it has one.
 template <int EST, int XP>
 __device__ __forceinline__ void stage_exact_table() {
-  if constexpr (EST != EST_APPROX && XP == XP_F32) stage_phi_inv();
+  if constexpr (EST != EST_APPROX && XP == XP_F32) stage_phi_inv(phi_inv_smem());
   if constexpr (EST != EST_APPROX && XP == XP_F64) stage_phi64();
 }
 
@@ -116,7 +116,8 @@ __device__ __forceinline__ int32_t ff_sum1(const FastFixed &ff, int32_t z, int32
 // reading bits [32 - d(L+1), 32 - dL) of the shared word (packed draws).
 // MSEL: 0 the item uses a table lookup (Methods 1 and 2), 1 the line
 // evaluation of Method 3, 2 either, chosen per step (only the per-sample
-// dump instantiation); chosen once per chunk, so the hot step code has no
+// dump instantiation), 4 a table lookup whose exact path is coupled by Method
+// 2's ranks (corrections); chosen once per chunk, so the hot step code has no
 // branch on the method.  FP64 exact kernels: 0 increments in 64-bit integers
 // (exact64.cuh), 1 in FP64.
 // PRE (merged nested kernel, family 24): the 32-bit fast datapath's sum1
@@ -134,6 +135,7 @@ struct LevelSim {
   static constexpr bool HAS_EXACT = (EST != EST_APPROX);
   static constexpr bool HAS_APPROX = (EST != EST_EXACT);
   static constexpr bool MIL = (SCHEME == 1);
+  static constexpr bool PERM = EST == EST_CORR && MSEL >= 2;   // Method 2's coupling of the exact path
   static constexpr bool FAST = (AP == AP_FX32 || AP == AP_FX64);
   static constexpr bool FIXED = (AP == AP_FIXED || FAST);
   static constexpr bool HALF = (AP == AP_F16 || AP == AP_BF16 || AP == AP_F16S || AP == AP_BF16S);
@@ -169,6 +171,7 @@ struct LevelSim {
   uint32_t rot[KP], off_mask;
   const uint16_t *perm_s;  // method 2 coupling of the exact path (shared memory), or nullptr
   const float4 *phi;       // FP32 exact path: the inverse-Normal cubics in shared memory
+  uint32_t phil;           // and this lane's copy (phi_lane)
   uint32_t low_mask;
   X c1, c2, c1c, c3, S0, K;
   // FP64 exact path: integer increments (exact64.cuh)
@@ -243,9 +246,12 @@ struct LevelSim {
       off_mask = ((1u << it.d) - 1u) << 3;
     }
     perm_s = nullptr;
-    if constexpr (HAS_EXACT && XP == XP_F32) phi = phi_inv_smem();
+    if constexpr (HAS_EXACT && XP == XP_F32) {
+      phi = phi_inv_smem();
+      phil = phi_lane();
+    }
     low_mask = (1u << dshift) - 1u;
-    if constexpr (EST == EST_CORR) {
+    if constexpr (PERM) {
       if (it.perm) perm_s = (const uint16_t *)((const unsigned char *)tab + ((size_t)1 << it.d) * TabBytes<AP>::value);
     }
   }
@@ -394,7 +400,7 @@ struct LevelSim {
   // Approximate Normal of J in Z's fixed-point format: Method 1 reads the
   // signed table at j = top d bits of J; Method 3 evaluates the class line.
   __device__ __forceinline__ int32_t fixed_z(uint32_t J) const {
-    if constexpr (MSEL == 0) return ((const int32_t *)smem_tab)[J >> dshift];
+    if constexpr (MSEL == 0 || MSEL == 4) return ((const int32_t *)smem_tab)[J >> dshift];
     if constexpr (MSEL == 2) {
       if (method != 3) return ((const int32_t *)smem_tab)[J >> dshift];
     }
@@ -411,7 +417,7 @@ struct LevelSim {
   }
 
   __device__ __forceinline__ H half_z(uint32_t J) const {
-    if constexpr (MSEL == 0) return HO::from_bits(((const uint16_t *)smem_tab)[J >> dshift]);
+    if constexpr (MSEL == 0 || MSEL == 4) return HO::from_bits(((const uint16_t *)smem_tab)[J >> dshift]);
     if constexpr (MSEL == 2) {
       if (method != 3) return HO::from_bits(((const uint16_t *)smem_tab)[J >> dshift]);
     }
@@ -433,7 +439,10 @@ struct LevelSim {
     if constexpr (HAS_EXACT) {
       // Method 2 (Sec. 3.2): the exact path takes the uniform in the interval
       // pi(j) that the approximate value of j is ranked at, with J's low bits
-      const uint32_t Je = perm_s ? (((uint32_t)perm_s[J >> dshift] << dshift) | (J & low_mask)) : J;
+      uint32_t Je = J;
+      if constexpr (PERM) {
+        if (MSEL != 2 || perm_s) Je = ((uint32_t)perm_s[J >> dshift] << dshift) | (J & low_mask);
+      }
       X z, inc;
       int64_t qi = 0;
       uint64_t y = 0;
@@ -452,7 +461,7 @@ struct LevelSim {
           inc = exact_inc(z, c1, X(1));
         }
       } else {
-        z = exact_normal_f32(Je, phi);
+        z = exact_normal_f32(Je, phi, phil);
         inc = exact_inc(z, c1, X(1));
       }
       if constexpr (PC == PC_ASIAN) { if (i > 0) accF = accF + S; }
@@ -691,19 +700,20 @@ struct LevelSim {
       acc.nsat += lsat;
       ydump = (double)yi * (double)unit_scale;
     } else {
-      if (!valid) return;
+      // a sample outside the item's range adds zero: no branch
       if constexpr (EST == EST_EXACT) {
-        const X y = pf - pc;
+        const X y = valid ? pf - pc : X(0);
         acc.add_real(y);
         ydump = (double)y;
       } else {
         const float yx = (float)(pf - pc);
         const float ya = __fmul_rn(__ll2float_rn(qf - qc), unit_scale);
-        const float y = __fsub_rn(yx, ya);
+        const float y = valid ? __fsub_rn(yx, ya) : 0.0f;
         acc.add_real(y);
         ydump = (double)y;
       }
-      acc.nsat += lsat;
+      acc.nsat += valid ? lsat : 0u;
+      if (!valid) return;
     }
     if (dump) {
       mlmc_sample_rec r;
@@ -778,13 +788,13 @@ struct ThreadAcc {
   __device__ __forceinline__ void rewind(const Mark &m) {
     isum = m.isum; q_lo = m.q_lo; q_hi = m.q_hi;
   }
-  // s + y = t + e exactly (Knuth's TwoSum, six FP32 operations); e goes to c.
-  static __device__ __forceinline__ void two_sum_into(float &s, float &c, float y) {
+  // s + y = t + e exactly (Knuth's TwoSum, six FP32 operations): s becomes t, e is returned.
+  static __device__ __forceinline__ float two_sum(float &s, float y) {
     const float t = __fadd_rn(s, y);
     const float z = __fsub_rn(t, s);
     const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(y, z));
     s = t;
-    c = __fadd_rn(c, e);
+    return e;
   }
   // A real sample.  FP64 samples are added in FP64.  An FP32 sample y enters
   // the float pair (fs, fc) by TwoSum, so fs + fc misses sum y only by the
@@ -803,15 +813,15 @@ struct ThreadAcc {
       dq = fma((double)y, (double)y, dq);
     } else {
       const float yf = (float)y;
-      two_sum_into(fs, fc, yf);
+      fc = __fadd_rn(fc, two_sum(fs, yf));
       const float p = __fmul_rn(yf, yf);
       const float pe = __fmaf_rn(yf, yf, -p);
-      two_sum_into(fs2, fc2, p);
-      fc2 = __fadd_rn(fc2, pe);
+      fc2 = __fadd_rn(__fadd_rn(fc2, two_sum(fs2, p)), pe);
     }
   }
+  static constexpr bool PAIRS = EST != EST_APPROX && !(XP == XP_F64 && EST == EST_EXACT);
   __device__ __forceinline__ void flush_real() {
-    if constexpr (!(XP == XP_F64 && EST == EST_EXACT) && EST != EST_APPROX) {
+    if constexpr (PAIRS) {
       ds += (double)fs;
       ds += (double)fc;
       dq += (double)fs2;
@@ -910,9 +920,10 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
     uint64_t qbase = P * calls;
     if constexpr (E && Sim::LAZY) opaque(qbase);
     sim.begin();
+    // qbase is a multiple of calls (a power of two): the calls share its high word
+    const PhiloxStream ps((uint32_t)(qbase >> 32), it.ctr2, it.ctr3, args.rk);
     for (uint32_t c = 0; c < calls; ++c) {
-      const uint64_t q = qbase + c;
-      const uint4 w = philox4x32_10(make_uint4((uint32_t)q, (uint32_t)(q >> 32), it.ctr2, it.ctr3), args.rk);
+      const uint4 w = ps.call((uint32_t)qbase + c, args.rk);
       const int i0 = (int)(c << 2);
       sim.template step<true, 0, E>(w.x << lsh, i0);
       sim.template step<true, 1, E>(w.y << lsh, i0 + 1);
@@ -1067,6 +1078,7 @@ __device__ __forceinline__ void group_loop(Sim &sim, ThreadAcc<EST, XP> &acc, co
       }
     }
   }
+  acc.flush_real();
 }
 
 // Simulate one chunk of an item (its table already in shared memory) and
@@ -1122,7 +1134,6 @@ __device__ __forceinline__ void chunk_body(const LaunchArgs &args, const ItemDes
     else if (lc == 1) loop(L1{}, PayTag<-1>{});
     else loop(L2{}, PayTag<-1>{});
   }
-  acc.flush_real();
   block_reduce_write<EST, XP>(acc, args.partials + gc);
   if (args.counters && threadIdx.x < 32) {
     // the CTA that completes the item's last chunk sums all its partials, in
@@ -1171,6 +1182,7 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
     }
     if (lane == 0) s_item = lo;
   }
+  copies_done();   // of the exact path's table, started before the first chunk
   __syncthreads();
   const int item = s_item;
   const ItemDesc &it = items[item];
@@ -1191,6 +1203,9 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
     const int32_t S0q = (int32_t)it.fx.S0, Kq = (int32_t)it.fx.K;
     const void *ztab = it.ztab;
     const int n = 1 << d;
+    // merged launch: only the correction chunks (kind 2) run the FP32 exact path;
+    // the copies proceed while the pairs are formed
+    if (PHI_BY_KIND && it.kind == 2) stage_phi_inv(phi_inv_smem());
     int2 *dst = (int2 *)smem_tab;
     const M3Coef *m3 = (const M3Coef *)ztab;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
@@ -1230,7 +1245,7 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
       for (int k = threadIdx.x; k < n; k += blockDim.x) pd[k] = it.perm[k];
     }
     // merged launch: only the correction chunks (kind 2) run the FP32 exact path
-    if (PHI_BY_KIND && it.kind == 2) stage_phi_inv();
+    copies_done();
     __syncthreads();
   } else if constexpr (AP != AP_NONE) {
     if (!staged || it.ztab != *staged) {
@@ -1274,16 +1289,22 @@ __device__ __forceinline__ void run_chunk(const LaunchArgs &args, const ItemDesc
     else chunk_body<EST, XP, AP, SCHEME, PC, KP, 1, false, DYN>(args, it, item, gc, smem_tab);
   } else if constexpr (AP == AP_NONE || AP == AP_FX32) {
     // no method choice: exact paths, and the FX32 table that holds every method's values
-    chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
+    if (EST == EST_CORR && it.perm) {
+      if constexpr (EST == EST_CORR) chunk_body<EST, XP, AP, SCHEME, PC, KP, 4, false, DYN>(args, it, item, gc, smem_tab);
+    } else {
+      chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
+    }
   } else {
-    if (it.method == 3) chunk_body<EST, XP, AP, SCHEME, PC, KP, 1, false, DYN>(args, it, item, gc, smem_tab);
+    if (EST == EST_CORR && it.perm) {
+      if constexpr (EST == EST_CORR) chunk_body<EST, XP, AP, SCHEME, PC, KP, 4, false, DYN>(args, it, item, gc, smem_tab);
+    } else if (it.method == 3) chunk_body<EST, XP, AP, SCHEME, PC, KP, 1, false, DYN>(args, it, item, gc, smem_tab);
     else chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
   }
 }
 
 // Static launch: CTA b runs chunk chunk0 + b of the launch.
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
-__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, AP, SCHEME, PC>::value)
+__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC>::value)
 level_kernel(const __grid_constant__ LaunchArgs args) {
   stage_exact_table<EST, XP>();
   run_chunk<EST, XP, AP, SCHEME, PC, KP, false, false>(args, args.items, args.n_items, args.chunk0 + blockIdx.x,
@@ -1294,7 +1315,7 @@ level_kernel(const __grid_constant__ LaunchArgs args) {
 // its own, so that the record-writing code does not weigh on the register
 // allocation of the launches without records.
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
-__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, AP, SCHEME, PC>::value)
+__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC>::value)
 level_kernel_dump(const __grid_constant__ LaunchArgs args) {
   stage_exact_table<EST, XP>();
   run_chunk<EST, XP, AP, SCHEME, PC, KP, true, false>(args, args.items, args.n_items, args.chunk0 + blockIdx.x,
@@ -1305,7 +1326,7 @@ level_kernel_dump(const __grid_constant__ LaunchArgs args) {
 // and chunk counts come from args.dyn, written on the device before the
 // launch; CTA b runs chunks b, b + gridDim.x, ...
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
-__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, AP, SCHEME, PC, true>::value)
+__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC, true>::value)
 level_kernel_dyn(const __grid_constant__ LaunchArgs args) {
   const DynLaunch d = *args.dyn;
   const void *staged = nullptr;
@@ -1332,6 +1353,8 @@ __global__ void __launch_bounds__(LAUNCH_THREADS, 6) nested_kernel(const __grid_
     chunk_body<EST_APPROX, XP_F32, AP, SCHEME, PC, 3, 0, false, false, PRE, true>(args, it, item, gc, smem_tab);
   else if (it.kind == 1)
     chunk_body<EST_APPROX, XP_F32, AP, SCHEME, PC, 1, 0, false, false, PRE, true>(args, it, item, gc, smem_tab);
+  else if (it.perm)
+    chunk_body<EST_CORR, XP_F32, AP, SCHEME, PC, 1, 4, false, false, PRE, true>(args, it, item, gc, smem_tab);
   else
     chunk_body<EST_CORR, XP_F32, AP, SCHEME, PC, 1, 0, false, false, PRE, true>(args, it, item, gc, smem_tab);
 }
@@ -1346,8 +1369,8 @@ cudaError_t launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t st, cons
             : a.dump       ? level_kernel_dump<EST, XP, AP, SCHEME, PC, KP>
                            : level_kernel<EST, XP, AP, SCHEME, PC, KP>;
   // above 48 KB of dynamic plus static shared memory (the static part holds
-  // up to about 8.6 KB: the inverse-Normal cubics) the kernel must opt in
-  if (smem > 32 * 1024) {
+  // up to about 19.6 KB: the inverse-Normal cubics) the kernel must opt in
+  if (smem > 24 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }

@@ -13,12 +13,14 @@ using namespace mlmc;
 namespace {
 
 __global__ void exact_normal_kernel(const uint32_t *J, float *z, uint64_t n) {
-  __shared__ float4 tab[PHI_INV_PARTS];
-  for (int k = threadIdx.x; k < PHI_INV_PARTS; k += blockDim.x) tab[k] = k_phi_inv[k];
+  __shared__ float4 tab[PHI_SMEM];
+  stage_phi_inv(tab);
+  copies_done();
   __syncthreads();
+  const uint32_t lane = phi_lane();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    z[i] = exact_normal_f32(J[i], tab);
+    z[i] = exact_normal_f32(J[i], tab, lane);
 }
 
 }  // namespace
