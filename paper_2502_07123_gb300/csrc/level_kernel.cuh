@@ -1135,19 +1135,31 @@ __device__ __forceinline__ void chunk_body(const LaunchArgs &args, const ItemDes
     else loop(L2{}, PayTag<-1>{});
   }
   block_reduce_write<EST, XP>(acc, args.partials + gc);
-  if (args.counters && threadIdx.x < 32) {
-    // the CTA that completes the item's last chunk sums all its partials, in
-    // chunk order (the partials of other CTAs are read through L2); only its
-    // first warp takes part, the other warps are done
+  if (!DYN && args.counters) {
+    // the CTA that completes the item's last chunk sums all its partials, in a
+    // fixed order; up to 32 of them (the other columns are empty: adding their
+    // zeros changes nothing) are one warp's work, without the CTA's barriers
+    const bool few = it.n_chunks <= 32u;
+    __shared__ uint32_t s_last;
     uint32_t last = 0;
     if (threadIdx.x == 0) {
       __threadfence();
       last = atomicAdd(args.counters + item, 1u) + 1u == it.n_chunks;
+      s_last = last;
     }
-    last = __shfl_sync(0xffffffffu, last, 0);
+    if (few) {
+      if (threadIdx.x < 32) last = __shfl_sync(0xffffffffu, last, 0);
+    }
+    else {
+      __syncthreads();
+      last = s_last;
+    }
     if (last) {
       __threadfence();
-      const DevSums r = warp_sum_partials<true>(args.partials + it.chunk_begin, it.n_chunks);
+      constexpr bool INTS = EST == EST_APPROX;
+      const Partial *p = args.partials + it.chunk_begin;
+      const DevSums r = few ? to_sums(group_sum<INTS, !INTS>(one_chunk<INTS, !INTS>(p, it.n_chunks, threadIdx.x)))
+                            : cta_sum_partials<INTS, !INTS>(p, it.n_chunks);
       if (threadIdx.x == 0) {
         args.out[it.out_index] = r;
         args.counters[item] = 0u;   // ready for the next launch
