@@ -173,6 +173,8 @@ bool lane_split(uint64_t N, int num_sms);
 bool sample_range_ok(int level, uint64_t first, uint64_t N);
 mlmc_status build_item(const mlmc_work &w, int out_index, void *dump, BuiltItem &b, double &disc, int &unit,
                        int &exact_int, TableSource &src);
+// An item's integer increments of the FP64 exact path (from its FP64 constants).
+void exact64_consts(mlmc::ItemDesc &it, bool milstein);
 // build_item through the per-process cache of built constants.
 mlmc_status build_item_cached(const mlmc_work &w, int out_index, void *dump, BuiltItem &b, double &disc, int &unit,
                               int &exact_int);

@@ -12,13 +12,20 @@
 // S_{k+1} = S_k (1 + sum1_k), d S_n / d S_{k+1} = S_n / S_{k+1}, so every
 // sensitivity is a_f S_n (resp. a_c S^c_m) times a per-step factor
 // (1 / S_{k+1}, 1 / (1 + sum1_k), Z_k / (1 + sum1_k), ...), where
-// a_f = e^{-rT} 1[S_n > K] and a_c = -e^{-rT} 1[S^c_m > K].  A thread
-// therefore needs no tape: pass 1 runs the sample forward and accumulates the
-// per-step factor sums (which give the per-type second moments once S_n and
-// S^c_m are known); pass 2 regenerates the same uniforms, forms each
-// instance's sensitivity and adds its square, summed over the warp, into the
-// warp's own shared-memory row (deterministic order).  Per-CTA partials are
-// summed in CTA order by sens_finalize_kernel.
+// a_f = e^{-rT} 1[S_n > K] and a_c = -e^{-rT} 1[S^c_m > K].
+//
+// FP64 operations (2 lanes per clock and SM here) are what the time goes to, so
+// there are as few of them as the statistics need.  A CTA takes 128 samples at a
+// time.  Pass 1, a thread per sample, runs both paths -- Normals and increments
+// in integers (exact64.cuh), one reciprocal u = 1 / (1 + sum1) per step, 1 / S
+// by 1 / S_{k+1} = u / S_k -- and writes u and 1 / S of every step to a tape in
+// global memory (32 bytes at a time; it stays in L2 up to level 6 or so).  Pass
+// 2, a thread per instance, adds the squares over the CTA's samples: no
+// cross-lane sums, and the tape read in rows.  The per-type moments are sums of
+// the per-instance ones.  About 40 FP64 operations per path-step against 258
+// (two library Phi^-1, four divisions, 64-bit butterflies): 100,001 level-6
+// samples 3.31 -> 0.49 ms, the FP64 unit 85% busy in both.
+// Per-CTA partials are summed in CTA order by sens_finalize_kernel.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -27,6 +34,7 @@
 #include <vector>
 
 #include "device_common.cuh"
+#include "exact64.cuh"
 #include "host_api.h"
 #include "item.h"
 #include "mlmc.h"
@@ -36,26 +44,21 @@ using namespace mlmc;
 namespace {
 
 constexpr int SENS_THREADS = 128;
-constexpr int SENS_WARPS = SENS_THREADS / 32;
 constexpr int SENS_MAX_LEVEL = 10;
-// per-instance rows kept on the device: S-type (= mul2 except S0), sum1-type (= mul1), Z
+// per-instance rows: S-type (= mul2 except S0), sum1-type (= mul1), Z
 constexpr int SENS_ROWS = 3;
 enum { T_Z = 0, T_CON1 = 1, T_CON2 = 2, T_MUL1 = 3, T_SUM1 = 4, T_MUL2 = 5, T_S = 6 };
+// per-CTA scalars: sums, then maxima
+enum { P_DP, P_DP2, P_C1F, P_C1C, P_C2, P_S0, P_SUMS, P_ZHI = P_SUMS, P_ZLO, P_ZCHI, P_ZCLO, P_MUL2, P_S, P_COUNT };
 
 struct SensConsts {
   double con1, con1c, con2, S0, K, disc;
   int level, n, m, ni;
   uint64_t first, N;
   uint32_t ctr2, ctr3;
-};
-
-// Per-CTA partial: per-type sums of squared sensitivities, maxima, DeltaP sums,
-// and the per-sample scalar instances (con1 fine / coarse, con2, S0).
-struct SensPartial {
-  double A[7];
-  double maxabs[7];
-  double sdp, sdp2;
-  double c1f, c1c, c2, s0;
+  int64_t q1;          // integer increments (exact64.cuh; qF 0: they may reach 8, formed in FP64)
+  uint64_t q2;
+  int qF;
 };
 
 __device__ __forceinline__ double warp_sum(double x) {
@@ -69,174 +72,246 @@ __device__ __forceinline__ double warp_max(double x) {
   return x;
 }
 
-// Exact FP64 Normal of fine step k of sample s (stream 0); `q` / `w` cache the
-// last Philox call of this thread.
-struct Draws {
-  uint64_t q = ~0ULL;
-  uint4 w;
-  __device__ __forceinline__ double z(const SensConsts &c, const RoundKeys &rk, uint64_t s, int k) {
-    const uint64_t wi = (s << c.level) + (uint64_t)k;
-    const uint64_t qq = wi >> 2;
-    if (qq != q) {
-      q = qq;
-      w = philox4x32_10(make_uint4((uint32_t)qq, (uint32_t)(qq >> 32), c.ctr2, c.ctr3), rk);
-    }
-    return exact_normal_f64(word_of(w, (int)(wi & 3)));
-  }
-};
+// 1 / x: the hardware's single-precision reciprocal r of x and one cubic step of
+// Newton's iteration, r (1 + e + e^2) with e = 1 - x r (|e| < 2^-21, so what is
+// left out is below 2^-63); by division outside the float range.
+__device__ __forceinline__ double reciprocal(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const uint32_t mag = (uint32_t)hi & 0x7FFFFFFFu;
+  if (mag - 0x39B00000u >= 0x0C800000u) return 1.0 / x;   // |x| outside [2^-100, 2^100)
+  const float f = __uint_as_float(((mag - 0x38000000u) << 3) | ((uint32_t)lo >> 29));
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+  const uint32_t b = __float_as_uint(rf);
+  const double r = __hiloint2double((int)(((b >> 3) + 0x38000000u) | ((uint32_t)hi & 0x80000000u)), (int)(b << 29));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
 
-__global__ void __launch_bounds__(SENS_THREADS) sens_kernel(const SensConsts c, const RoundKeys rk, int iters,
-                                                            SensPartial *part, double *inst_part) {
-  extern __shared__ double srow[];   // [warp][SENS_ROWS][ni]
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int ni = c.ni, n = c.n, m = c.m;
-  double *row = srow + (size_t)warp * SENS_ROWS * ni;
-  for (int i = lane; i < SENS_ROWS * ni; i += 32) row[i] = 0.0;
-  __syncwarp();
-  double A[7] = {0, 0, 0, 0, 0, 0, 0}, mx[7] = {0, 0, 0, 0, 0, 0, 0};
-  double sdp = 0.0, sdp2 = 0.0, c1f = 0.0, c1c = 0.0, c2s = 0.0, s0s = 0.0;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+// The larger of |x| and the running maximum m >= 0, by integer comparison (a NaN loses).
+__device__ __forceinline__ void max_abs(double &m, double x) {
+  const long long b = __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFLL;
+  if (b > __double_as_longlong(m) && b <= 0x7FF0000000000000LL) m = __longlong_as_double(b);
+}
+
+// Tape of a CTA's 128 samples: u and 1 / S of the fine steps [sample][n], then of
+// the coarse steps [sample][m].
+__host__ __device__ inline size_t tape_doubles(int n, int m) { return (size_t)SENS_THREADS * 2 * (n + m); }
+// Accumulators of pass 2 in shared memory: 3 fine rows of max(n, 128) and 2
+// coarse rows of max(m, 128) (below 128 instances several threads share one,
+// each with the samples of its residue).
+__host__ __device__ inline int slots(int n) { return n > SENS_THREADS ? n : SENS_THREADS; }
+
+__global__ void __launch_bounds__(SENS_THREADS, 4) sens_kernel(const SensConsts c, const RoundKeys rk, int iters,
+                                                            double *part, double *inst_part, double *tapes) {
+  extern __shared__ double acc[];
+  __shared__ double sF[SENS_THREADS], sG[SENS_THREADS], wp[P_COUNT][SENS_THREADS / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int n = c.n, m = c.m, nf = slots(n), nc = m > 0 ? slots(m) : 0;
+  double *fine = acc, *coarse = acc + 3 * nf;
+  for (int i = tid; i < 3 * nf + 2 * nc; i += SENS_THREADS) acc[i] = 0.0;
+  stage_phi64();
+  copies_done();
+  __syncthreads();
+  const ulonglong2 *phi = phi64_smem();
+  double *tu = tapes + tape_doubles(n, m) * blockIdx.x, *tr = tu + (size_t)SENS_THREADS * n;
+  double *tv = tr + (size_t)SENS_THREADS * n, *tw = tv + (size_t)SENS_THREADS * m;
+  const uint32_t qhi = (uint32_t)(1085 - c.qF) << 20, zhi0 = (uint32_t)(1085 - 59) << 20;
+  const double rS0 = 1.0 / c.S0;
+  double ps[P_SUMS] = {0, 0, 0, 0, 0, 0}, mm2 = 0.0, mS = c.S0;
+  // extremes of Z (units 2^-59) on the fine and the coarse path; a lane without a
+  // sample of its own repeats sample `first`, which changes no extreme
+  long long z_hi = -0x7FFFFFFFFFFFFFFFLL, z_lo = 0x7FFFFFFFFFFFFFFFLL, zc_hi = z_hi, zc_lo = z_lo;
+  const uint64_t stride = (uint64_t)gridDim.x * SENS_THREADS;
   for (int it = 0; it < iters; ++it) {
-    const uint64_t rel = (uint64_t)it * stride + (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t rel = (uint64_t)it * stride + (uint64_t)blockIdx.x * SENS_THREADS + tid;
     const bool valid = rel < c.N;
     const uint64_t s = c.first + (valid ? rel : 0);
-    // ---- pass 1: forward, factor sums ----
-    Draws dr;
-    double S = c.S0, Sc = c.S0, zprev = 0.0;
-    double inv2S = 0.0, u2 = 0.0, u1 = 0.0, zu = 0.0;
-    double inv2Sc = 0.0, v2 = 0.0, v1 = 0.0, zcv = 0.0, uv = 0.0, uprev = 0.0;
-    double mz = 0.0, m1 = 0.0, ms1 = 0.0, mm2 = 0.0, mS = c.S0;
-    for (int k = 0; k < n; ++k) {
-      const double z = dr.z(c, rk, s, k);
-      const double mul1 = c.con2 * z;
-      const double sum1 = c.con1 + mul1;
-      const double mul2 = S * sum1;
-      S = S + mul2;
-      const double u = 1.0 / (1.0 + sum1);
-      inv2S += 1.0 / (S * S);
-      u2 += u * u;
-      u1 += u;
-      zu += z * u;
-      mz = fmax(mz, fabs(z)); m1 = fmax(m1, fabs(mul1)); ms1 = fmax(ms1, fabs(sum1));
-      mm2 = fmax(mm2, fabs(mul2)); mS = fmax(mS, fabs(S));
-      if (m > 0 && (k & 1)) {
-        const double zc = zprev + z;
-        const double mul1c = c.con2 * zc;
-        const double sum1c = c.con1c + mul1c;
-        const double mul2c = Sc * sum1c;
-        Sc = Sc + mul2c;
-        const double v = 1.0 / (1.0 + sum1c);
-        inv2Sc += 1.0 / (Sc * Sc);
-        v2 += v * v;
-        v1 += v;
-        zcv += zc * v;
-        uv += v * (uprev + u);
-        m1 = fmax(m1, fabs(mul1c)); ms1 = fmax(ms1, fabs(sum1c));
-        mm2 = fmax(mm2, fabs(mul2c)); mS = fmax(mS, fabs(Sc));
-      }
-      zprev = z;
-      uprev = u;
-    }
-    const double Pf = c.disc * (S > c.K ? S - c.K : 0.0);
-    const double Pc = m > 0 ? c.disc * (Sc > c.K ? Sc - c.K : 0.0) : 0.0;
-    const double F = valid && S > c.K ? c.disc * S : 0.0;
-    const double G = valid && m > 0 && Sc > c.K ? -c.disc * Sc : 0.0;
-    if (valid) {
-      const double dp = Pf - Pc;
-      sdp += dp;
-      sdp2 += dp * dp;
-      mx[T_Z] = fmax(mx[T_Z], mz); mx[T_MUL1] = fmax(mx[T_MUL1], m1); mx[T_SUM1] = fmax(mx[T_SUM1], ms1);
-      mx[T_MUL2] = fmax(mx[T_MUL2], mm2); mx[T_S] = fmax(mx[T_S], mS);
-    }
-    const double sS0 = (F + G) / c.S0;
-    A[T_S] += F * F * inv2S + G * G * inv2Sc + sS0 * sS0;
-    A[T_MUL2] += F * F * inv2S + G * G * inv2Sc;
-    A[T_SUM1] += F * F * u2 + G * G * v2;
-    A[T_MUL1] += F * F * u2 + G * G * v2;
-    const double a1f = F * u1, a1c = G * v1, a2 = F * zu + G * zcv;
-    A[T_CON1] += a1f * a1f + a1c * a1c;
-    A[T_CON2] += a2 * a2;
-    A[T_Z] += c.con2 * c.con2 * (F * F * u2 + 2.0 * F * G * uv + 2.0 * G * G * v2);
-    c1f += a1f * a1f; c1c += a1c * a1c; c2s += a2 * a2; s0s += sS0 * sS0;
-    // ---- pass 2: per-instance squares (same uniforms), summed over the warp ----
-    Draws dr2;
-    S = c.S0; Sc = c.S0; zprev = 0.0; uprev = 0.0;
-    for (int k = 0; k < n; ++k) {
-      const double z = dr2.z(c, rk, s, k);
-      const double sum1 = c.con1 + c.con2 * z;
-      S = S + S * sum1;
-      const double u = 1.0 / (1.0 + sum1);
-      const double xs = F / S, xu = F * u;
-      const double ws = warp_sum(xs * xs), wu = warp_sum(xu * xu);
-      if (lane == 0) { row[k] += ws; row[ni + k] += wu; }
-      if (m > 0 && (k & 1)) {
-        const double zc = zprev + z;
-        const double sum1c = c.con1c + c.con2 * zc;
-        Sc = Sc + Sc * sum1c;
-        const double v = 1.0 / (1.0 + sum1c);
-        const int kc = k >> 1;
-        const double ys = G / Sc, yv = G * v;
-        const double za = c.con2 * (F * uprev + G * v), zb = c.con2 * (F * u + G * v);
-        const double w1 = warp_sum(ys * ys), w2 = warp_sum(yv * yv), w3 = warp_sum(za * za), w4 = warp_sum(zb * zb);
-        if (lane == 0) {
-          row[n + kc] += w1; row[ni + n + kc] += w2;
-          row[2 * ni + k - 1] += w3; row[2 * ni + k] += w4;
+    // ---- pass 1: both paths, u and 1 / S of every step to the tape ----
+    double S = c.S0, Sc = c.S0, r = rS0, rc = rS0, u1 = 0.0, zu = 0.0, v1 = 0.0, zcv = 0.0;
+    long long zprev = 0, qprev = 0;
+    // one step of a path from its Normal zq 2^-59 and increment q 2^-qF
+    auto advance = [&](long long zq, long long q, double con1, double &St, double &rt, double &a1, double &az) {
+      const double z = q_to_double(zq, zhi0);
+      const double sum1 = c.qF ? q_to_double(q, qhi) : fma(c.con2, z, con1);
+      const double mul2 = St * sum1;
+      St = St + mul2;
+      const double u = reciprocal(1.0 + sum1);
+      rt *= u;
+      a1 += u;
+      az = fma(z, u, az);
+      max_abs(mm2, mul2);
+      max_abs(mS, St);
+      return u;
+    };
+    for (int k0 = 0; k0 < n; k0 += 4) {
+      const uint64_t wi = (s << c.level) + (uint64_t)k0;
+      const uint4 w = philox4x32_10(make_uint4((uint32_t)(wi >> 2), (uint32_t)(wi >> 34), c.ctr2, c.ctr3), rk);
+      double us[4], rs[4], vs[2], ws[2];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (k0 + j >= n) break;
+        const uint32_t J = word_of(w, (int)((wi + j) & 3));
+        const int32_t mk = (int32_t)J >> 31;   // Z = y in the upper half, -y below
+        const uint64_t y = probit_q60(J ^ (uint32_t)mk, phi);
+        const long long zq = mk ? (long long)(y >> 1) : -(long long)(y >> 1);
+        const long long q = c.q1 + (long long)(mulhi64_3(c.q2, y) ^ (uint64_t)(int64_t)~mk);
+        z_hi = max(z_hi, zq);
+        z_lo = min(z_lo, zq);
+        us[j] = advance(zq, q, c.con1, S, r, u1, zu);
+        rs[j] = r;
+        if (m > 0 && (j & 1)) {
+          const long long zc = zprev + zq;
+          zc_hi = max(zc_hi, zc);
+          zc_lo = min(zc_lo, zc);
+          vs[j >> 1] = advance(zc, qprev + q, c.con1c, Sc, rc, v1, zcv);
+          ws[j >> 1] = rc;
         }
-      } else if (m == 0) {
-        const double zb = c.con2 * F * u;
-        const double w4 = warp_sum(zb * zb);
-        if (lane == 0) row[2 * ni + k] += w4;
+        zprev = zq;
+        qprev = q;
       }
-      zprev = z;
-      uprev = u;
+      const size_t f = (size_t)tid * n + k0, g = (size_t)tid * m + (k0 >> 1);
+      if (n >= 4) {
+        *(double2 *)(tu + f) = make_double2(us[0], us[1]);
+        *(double2 *)(tu + f + 2) = make_double2(us[2], us[3]);
+        *(double2 *)(tr + f) = make_double2(rs[0], rs[1]);
+        *(double2 *)(tr + f + 2) = make_double2(rs[2], rs[3]);
+        *(double2 *)(tv + g) = make_double2(vs[0], vs[1]);
+        *(double2 *)(tw + g) = make_double2(ws[0], ws[1]);
+      } else {
+        tu[f] = us[0];
+        tr[f] = rs[0];
+        if (n == 2) {
+          tu[f + 1] = us[1];
+          tr[f + 1] = rs[1];
+          tv[g] = vs[0];
+          tw[g] = ws[0];
+        }
+      }
     }
+    const bool inF = valid && S > c.K, inG = valid && m > 0 && Sc > c.K;
+    const double F = inF ? c.disc * S : 0.0, G = inG ? -c.disc * Sc : 0.0;
+    sF[tid] = F;
+    sG[tid] = G;
+    const double dp = (inF ? c.disc * (S - c.K) : 0.0) - (inG ? c.disc * (Sc - c.K) : 0.0);
+    const double a1f = F * u1, a1c = G * v1, a2 = fma(F, zu, G * zcv), sS0 = (F + G) * rS0;
+    ps[P_DP] += dp;
+    ps[P_DP2] = fma(dp, dp, ps[P_DP2]);
+    ps[P_C1F] = fma(a1f, a1f, ps[P_C1F]);
+    ps[P_C1C] = fma(a1c, a1c, ps[P_C1C]);
+    ps[P_C2] = fma(a2, a2, ps[P_C2]);
+    ps[P_S0] = fma(sS0, sS0, ps[P_S0]);
+    __syncthreads();
+    // ---- pass 2: a thread per instance (several, each with a residue of the samples, below 128) ----
+    for (int i = tid; i < nf; i += SENS_THREADS) {
+      const int k = i & (n - 1), step = nf / n;
+      double a0 = 0.0, a1 = 0.0, a2s = 0.0;
+      for (int t = i / n; t < SENS_THREADS; t += step) {
+        const double Ft = sF[t];
+        const double a = Ft * tr[(size_t)t * n + k], b = Ft * tu[(size_t)t * n + k];
+        const double z = m > 0 ? fma(sG[t], tv[(size_t)t * m + (k >> 1)], b) : b;
+        a0 = fma(a, a, a0);
+        a1 = fma(b, b, a1);
+        a2s = fma(z, z, a2s);
+      }
+      fine[i] += a0;
+      fine[nf + i] += a1;
+      fine[2 * nf + i] += a2s;
+    }
+    for (int i = tid; i < nc; i += SENS_THREADS) {
+      const int k = i & (m - 1), step = nc / m;
+      double a0 = 0.0, a1 = 0.0;
+      for (int t = i / m; t < SENS_THREADS; t += step) {
+        const double Gt = sG[t];
+        const double a = Gt * tw[(size_t)t * m + k], b = Gt * tv[(size_t)t * m + k];
+        a0 = fma(a, a, a0);
+        a1 = fma(b, b, a1);
+      }
+      coarse[i] += a0;
+      coarse[nc + i] += a1;
+    }
+    __syncthreads();
   }
   // ---- CTA reduction (warp order) ----
-  __shared__ SensPartial wp[SENS_WARPS];
-  SensPartial p;
-  for (int t = 0; t < 7; ++t) { p.A[t] = warp_sum(A[t]); p.maxabs[t] = warp_max(mx[t]); }
-  p.sdp = warp_sum(sdp); p.sdp2 = warp_sum(sdp2);
-  p.c1f = warp_sum(c1f); p.c1c = warp_sum(c1c); p.c2 = warp_sum(c2s); p.s0 = warp_sum(s0s);
-  if (lane == 0) wp[warp] = p;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    SensPartial t = wp[0];
-    for (int w = 1; w < SENS_WARPS; ++w) {
-      for (int q = 0; q < 7; ++q) { t.A[q] += wp[w].A[q]; t.maxabs[q] = fmax(t.maxabs[q], wp[w].maxabs[q]); }
-      t.sdp += wp[w].sdp; t.sdp2 += wp[w].sdp2;
-      t.c1f += wp[w].c1f; t.c1c += wp[w].c1c; t.c2 += wp[w].c2; t.s0 += wp[w].s0;
-    }
-    t.maxabs[T_CON1] = fmax(fabs(c.con1), m > 0 ? fabs(c.con1c) : 0.0);
-    t.maxabs[T_CON2] = fabs(c.con2);
-    part[blockIdx.x] = t;
+  const double zs = 0x1p-59, cs = m > 0 ? zs : 0.0;
+  const double mx[P_COUNT - P_SUMS] = {(double)z_hi * zs,  -(double)z_lo * zs, (double)zc_hi * cs,
+                                       -(double)zc_lo * cs, mm2,                mS};
+#pragma unroll
+  for (int t = 0; t < P_COUNT; ++t) {
+    const double x = t < P_SUMS ? warp_sum(ps[t < P_SUMS ? t : 0]) : warp_max(mx[t < P_SUMS ? 0 : t - P_SUMS]);
+    if (lane == 0) wp[t][warp] = x;
   }
-  double *out = inst_part + (size_t)blockIdx.x * SENS_ROWS * ni;
-  for (int i = threadIdx.x; i < SENS_ROWS * ni; i += blockDim.x) {
+  __syncthreads();
+  if (tid < P_COUNT) {
+    double x = wp[tid][0];
+    for (int w = 1; w < SENS_THREADS / 32; ++w) x = tid < P_SUMS ? x + wp[tid][w] : fmax(x, wp[tid][w]);
+    part[(size_t)blockIdx.x * P_COUNT + tid] = x;
+  }
+  double *out = inst_part + (size_t)blockIdx.x * SENS_ROWS * c.ni;
+  for (int i = tid; i < SENS_ROWS * c.ni; i += SENS_THREADS) {
+    const int row = i / c.ni, k = i - row * c.ni;
     double x = 0.0;
-    for (int w = 0; w < SENS_WARPS; ++w) x += srow[(size_t)w * SENS_ROWS * ni + i];
+    if (k < n)
+      for (int j = k; j < nf; j += n) x += fine[row * nf + j];
+    else if (k < n + m && row < 2)
+      for (int j = k - n; j < nc; j += m) x += coarse[row * nc + j];
     out[i] = x;
   }
 }
 
-// Sum the CTA partials in CTA order: block 0 the scalars, the others one
-// per-instance entry per thread.
-__global__ void sens_finalize_kernel(const SensPartial *part, const double *inst_part, int n_ctas, int ni,
-                                     SensPartial *res, double *inst) {
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    SensPartial t = part[0];
-    for (int b = 1; b < n_ctas; ++b) {
-      for (int q = 0; q < 7; ++q) { t.A[q] += part[b].A[q]; t.maxabs[q] = fmax(t.maxabs[q], part[b].maxabs[q]); }
-      t.sdp += part[b].sdp; t.sdp2 += part[b].sdp2;
-      t.c1f += part[b].c1f; t.c1c += part[b].c1c; t.c2 += part[b].c2; t.s0 += part[b].s0;
-    }
-    *res = t;
-  }
-  const int i = (blockIdx.x - 1) * blockDim.x + threadIdx.x;
-  if (blockIdx.x == 0 || i >= SENS_ROWS * ni) return;
-  double x = 0.0;
-  for (int b = 0; b < n_ctas; ++b) x += inst_part[(size_t)b * SENS_ROWS * ni + i];
-  inst[i] = x;
+// The CTA partials' totals, a warp per value (lane l adds CTAs l, l + 32, ..., then
+// a butterfly): P_COUNT scalars, then the rows.
+__global__ void sens_finalize_kernel(const double *part, const double *inst_part, int n_ctas, int rows, double *res) {
+  const int v = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (v >= P_COUNT + rows) return;
+  const double *p = v < P_COUNT ? part + v : inst_part + (v - P_COUNT);
+  const size_t pitch = v < P_COUNT ? P_COUNT : rows;
+  const bool is_max = v >= P_SUMS && v < P_COUNT;
+  double x = is_max ? -1e300 : 0.0;
+  for (int b = lane; b < n_ctas; b += 32) x = is_max ? fmax(x, p[b * pitch]) : x + p[b * pitch];
+  x = is_max ? warp_max(x) : warp_sum(x);
+  if (lane == 0) res[v] = x;
 }
+
+// Device workspace and pinned result staging, kept between calls (under the
+// library lock, each call synchronises): up to SENS_KEEP bytes, more is given
+// back at the end of the call.
+constexpr size_t SENS_KEEP = (size_t)128 << 20, SENS_MAX_TAPE = (size_t)1 << 30;
+struct SensSpace {
+  int device = -1;
+  char *d = nullptr;
+  size_t cap = 0;
+  double *h = nullptr;
+  size_t h_cap = 0;
+  bool reserve(int dev, size_t bytes, size_t h_doubles) {
+    if (d && (dev != device || bytes > cap)) release();
+    if (!d) {
+      if (cudaMalloc(&d, bytes) != cudaSuccess) {
+        d = nullptr;
+        return false;
+      }
+      cap = bytes;
+      device = dev;
+    }
+    if (h_doubles > h_cap) {
+      if (h) cudaFreeHost(h);
+      h = nullptr;
+      h_cap = 0;
+      if (cudaHostAlloc((void **)&h, sizeof(double) * h_doubles, cudaHostAllocDefault) != cudaSuccess) {
+        h = nullptr;
+        return false;
+      }
+      h_cap = h_doubles;
+    }
+    return true;
+  }
+  void release() {
+    if (d) cudaFree(d);
+    d = nullptr;
+    cap = 0;
+  }
+};
+SensSpace g_sens;
 
 }  // namespace
 
@@ -268,43 +343,46 @@ extern "C" mlmc_status mlmc_sensitivities(int level, uint64_t N, const mlmc_para
   c.ctr3 = p->request_id;
   RoundKeys rk;
   make_round_keys(seed, rk);
-  const int n_ctas = (int)std::min<uint64_t>((uint64_t)2 * ctx_num_sms(),
-                                             (N + SENS_THREADS - 1) / SENS_THREADS);
+  {
+    ItemDesc it;
+    std::memset(&it, 0, sizeof it);
+    it.level = level;
+    it.c1d = c.con1; it.c1cd = c.con1c; it.c2d = c.con2;
+    exact64_consts(it, false);
+    c.q1 = it.q1; c.q2 = it.q2; c.qF = it.qF;
+  }
+  // four CTAs per SM where the tape allows
+  const size_t tape = sizeof(double) * tape_doubles(c.n, c.m);
+  const uint64_t want = std::min<uint64_t>((uint64_t)4 * ctx_num_sms(), SENS_MAX_TAPE / tape);
+  const int n_ctas = (int)std::min<uint64_t>(want, (N + SENS_THREADS - 1) / SENS_THREADS);
   const uint64_t per = (uint64_t)n_ctas * SENS_THREADS;
   const int iters = (int)((N + per - 1) / per);
-  const size_t smem = sizeof(double) * SENS_WARPS * SENS_ROWS * (size_t)c.ni;
+  const size_t smem = sizeof(double) * (3 * (size_t)slots(c.n) + (c.m > 0 ? 2 * (size_t)slots(c.m) : 0));
   cudaStream_t st = ctx_stream();
-  SensPartial *d_part = nullptr, *d_res = nullptr;
-  double *d_ip = nullptr, *d_inst = nullptr;
-  const size_t rows = (size_t)SENS_ROWS * c.ni;
-  if (cudaMalloc(&d_part, sizeof(SensPartial) * n_ctas) != cudaSuccess ||
-      cudaMalloc(&d_res, sizeof(SensPartial)) != cudaSuccess ||
-      cudaMalloc(&d_ip, sizeof(double) * rows * n_ctas) != cudaSuccess ||
-      cudaMalloc(&d_inst, sizeof(double) * rows) != cudaSuccess) {
-    cudaFree(d_part); cudaFree(d_res); cudaFree(d_ip); cudaFree(d_inst);
-    return MLMC_ENOMEM;
-  }
+  const size_t rows = (size_t)SENS_ROWS * c.ni, n_res = P_COUNT + rows;
+  int dev = 0;
+  MLMC_CK(cudaGetDevice(&dev));
+  const size_t doubles = (size_t)n_ctas * (P_COUNT + rows) + n_res;
+  const size_t bytes = (size_t)n_ctas * tape + sizeof(double) * doubles;
+  if (!g_sens.reserve(dev, bytes, n_res)) return MLMC_ENOMEM;
+  double *d_tape = (double *)g_sens.d, *d_part = d_tape + (size_t)n_ctas * (tape / sizeof(double));
+  double *d_ip = d_part + (size_t)n_ctas * P_COUNT, *d_res = d_ip + (size_t)n_ctas * rows;
   mlmc_status rs = MLMC_OK;
-  SensPartial h_res;
-  std::vector<double> rowsum(rows);
-  do {
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(sens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-      rs = MLMC_ECUDA;
-      break;
-    }
-    sens_kernel<<<n_ctas, SENS_THREADS, smem, st>>>(c, rk, iters, d_part, d_ip);
-    sens_finalize_kernel<<<1 + (unsigned)((rows + 127) / 128), 128, 0, st>>>(d_part, d_ip, n_ctas, c.ni, d_res,
-                                                                             d_inst);
+  if (smem > 24 * 1024 &&
+      cudaFuncSetAttribute(sens_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+    rs = MLMC_ECUDA;
+  if (rs == MLMC_OK) {
+    sens_kernel<<<n_ctas, SENS_THREADS, smem, st>>>(c, rk, iters, d_part, d_ip, d_tape);
+    sens_finalize_kernel<<<(unsigned)((n_res + 3) / 4), 128, 0, st>>>(d_part, d_ip, n_ctas, (int)rows, d_res);
     if (cudaGetLastError() != cudaSuccess ||
-        cudaMemcpyAsync(&h_res, d_res, sizeof h_res, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaMemcpyAsync(rowsum.data(), d_inst, sizeof(double) * rows, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaMemcpyAsync(g_sens.h, d_res, sizeof(double) * n_res, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
       rs = MLMC_ECUDA;
-  } while (0);
-  cudaFree(d_part); cudaFree(d_res); cudaFree(d_ip); cudaFree(d_inst);
+  }
+  if (g_sens.cap > SENS_KEEP) g_sens.release();
   if (rs != MLMC_OK) return rs;
   // per-instance second moments, type-major 7 x ni
+  const double *res = g_sens.h, *rowsum = g_sens.h + P_COUNT;
   const int ni = c.ni, n = c.n, m = c.m;
   std::vector<double> E((size_t)7 * ni, 0.0);
   const double inv = 1.0 / (double)N;
@@ -314,21 +392,34 @@ extern "C" mlmc_status mlmc_sensitivities(int level, uint64_t N, const mlmc_para
     E[(size_t)T_SUM1 * ni + i] = rowsum[ni + i] * inv;
     E[(size_t)T_MUL1 * ni + i] = rowsum[ni + i] * inv;
   }
-  for (int j = 0; j < n; ++j) E[(size_t)T_Z * ni + j] = rowsum[2 * ni + j] * inv;
-  E[(size_t)T_S * ni + n + m] = h_res.s0 * inv;
-  E[(size_t)T_CON1 * ni + 0] = h_res.c1f * inv;
-  E[(size_t)T_CON1 * ni + 1] = h_res.c1c * inv;
-  E[(size_t)T_CON2 * ni + 0] = h_res.c2 * inv;
+  for (int j = 0; j < n; ++j) E[(size_t)T_Z * ni + j] = c.con2 * c.con2 * rowsum[2 * ni + j] * inv;
+  E[(size_t)T_S * ni + n + m] = res[P_S0] * inv;
+  E[(size_t)T_CON1 * ni + 0] = res[P_C1F] * inv;
+  E[(size_t)T_CON1 * ni + 1] = res[P_C1C] * inv;
+  E[(size_t)T_CON2 * ni + 0] = res[P_C2] * inv;
   std::memset(out, 0, sizeof *out);
-  for (int t = 0; t < 7; ++t) {
-    out->A[t] = h_res.A[t] * inv;
-    out->maxabs[t] = h_res.maxabs[t];
-    double b = 0.0;
-    for (int i = 0; i < ni; ++i) b += std::sqrt(E[(size_t)t * ni + i]);
-    out->B[t] = b;
+  // maxima: sum1 and mul1 are monotone in Z, so its extremes give theirs
+  auto larger = [](double a, double b) { return std::max(std::fabs(a), std::fabs(b)); };
+  const double zh = res[P_ZHI], zl = -res[P_ZLO], ch = res[P_ZCHI], cl = -res[P_ZCLO];
+  double mul1 = c.con2 * larger(zh, zl), sum1 = larger(c.con1 + c.con2 * zh, c.con1 + c.con2 * zl);
+  if (m > 0) {
+    mul1 = std::max(mul1, c.con2 * larger(ch, cl));
+    sum1 = std::max(sum1, larger(c.con1c + c.con2 * ch, c.con1c + c.con2 * cl));
   }
-  out->mean = h_res.sdp * inv;
-  out->var = std::max(0.0, h_res.sdp2 * inv - out->mean * out->mean);
+  const double mx[7] = {larger(zh, zl), larger(c.con1, m > 0 ? c.con1c : 0.0), std::fabs(c.con2), mul1, sum1,
+                        res[P_MUL2], res[P_S]};
+  for (int t = 0; t < 7; ++t) {
+    double a = 0.0, b = 0.0;
+    for (int i = 0; i < ni; ++i) {
+      a += E[(size_t)t * ni + i];
+      b += std::sqrt(E[(size_t)t * ni + i]);
+    }
+    out->A[t] = a;
+    out->B[t] = b;
+    out->maxabs[t] = mx[t];
+  }
+  out->mean = res[P_DP] * inv;
+  out->var = std::max(0.0, res[P_DP2] * inv - out->mean * out->mean);
   out->n = N;
   out->n_instances = ni;
   if (inst_out) std::memcpy(inst_out, E.data(), sizeof(double) * E.size());
