@@ -60,9 +60,10 @@ struct FastFixed {
   int64_t limT;              // lazy runs: S after an odd fine step (and the coarse S) at most limT
                              // keeps every fine S within lim_S (fast_fixed)
   int32_t lazy;              // 32-bit S may run unclamped, checked once per pack (fast_fixed)
-  int32_t pre_ok;            // |sum1| < 2^(rs2 - 1): sum1 2^(32 - rs2) fits 32 bits, so the rounded
-                             // product S sum1 is the high word of one 64-bit multiply-add
-                             // (the merged nested kernel's pre-scaled form, family 24)
+  int32_t pre_ok;            // the item takes the pre-scaled form (fast_fixed; LevelSim's PRE): sum1 2^(32 - rs2)
+                             // fits 32 bits, so the rounded product S sum1 is the high word of one 64-bit
+                             // multiply-add, sum1 is mul1 plus a constant, and for Euler-Maruyama the table
+                             // holds con2 Z~_j + radd1 in 4 bytes
 };
 
 struct ItemDesc {
@@ -85,8 +86,8 @@ struct ItemDesc {
   int32_t kind;            // in a merged nested launch: 0 approximate packed, 1 approximate one
                            // sample per thread, 2 correction (nested_kernel)
   int32_t tab_y0;          // 1: a level-0 approximate item of the 32-bit fast datapath with a terminal
-                           // payoff; its shared-memory table holds (Y_j, saturated_j), the sample value
-                           // of every index j (its one fine step is a function of j alone)
+                           // payoff; its shared-memory table holds Y_j, the sample value of every
+                           // index j (its one fine step is a function of j alone)
   float unit_scale;        // 2^-unit (FP32, correction estimators)
   // exact path constants
   float c1f, c2f, c1cf, c3f, S0f, Kf;

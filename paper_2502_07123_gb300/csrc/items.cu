@@ -323,10 +323,15 @@ bool fast_fixed(const int e[7], const int f[7], int64_t con1, int64_t con1c, int
   ff.rs1 = rs1; ff.rs3 = rs3; ff.rs_sum1 = rs_sum1; ff.rs2 = rs2 + k2;
   ff.mulS = 1 << shS;
   ff.radd1 = (int64_t)r1; ff.radd3 = (int64_t)r3; ff.radd2 = (int64_t)radd2;
-  // the pre-scaled product: sum1 2^(32 - rs2) and radd2 2^(32 - rs2) in range,
-  // |S| < 2^31 (32-bit S) so the 64-bit product cannot overflow
+  // the pre-scaled form (level_kernel.cuh, LevelSim's PRE): sum1 2^(32 - rs2) and
+  // radd2 2^(32 - rs2) in range, |S| < 2^31 (32-bit S) so the 64-bit product
+  // cannot overflow; mul1 on sum1's grid (con1's alignment and sum1's rounding
+  // cancel: every default format), so that sum1 = mul1 (+ mul3) + a constant; and
+  // for Euler the table's P_j = con2 Z~_j + radd1, and the coarse step's
+  // P_j + P_j' - radd1, in 32 bits
   const int rs2t = rs2 + k2;
-  ff.pre_ok = rs2t >= 1 && rs2t <= 31 && sum1_abs < ((I)1 << (rs2t - 1)) && radd2 < ((I)1 << 31);
+  ff.pre_ok = rs2t >= 1 && rs2t <= 31 && sum1_abs < ((I)1 << (rs2t - 1)) && radd2 < ((I)1 << 31) &&
+              shF1 == rs_sum1 && rs1 <= 31 && (milstein ? rs3 <= 31 : (I)con2 * zc + r1 < ((I)1 << 31));
   ff.mfine = (int64_t)1 << (2 * fZ);
   ff.mcoarse = (int64_t)2 << (2 * fZ);
   ff.limS = (int64_t)limS;
@@ -598,6 +603,7 @@ mlmc_status build_item(const mlmc_work &w, int out_index, void *dump, BuiltItem 
       const uint16_t *perm = nullptr;
       if ((s = src.m2_perm(p->icdf_bits, m2_fields_of(p), &perm)) != MLMC_OK) return s;
       it.perm = perm;
+      it.ff.pre_ok = 0;   // the coupled exact path runs beside the plain form only
       b.smem += sizeof(uint16_t) << p->icdf_bits;
     }
   }

@@ -53,16 +53,20 @@ constexpr int MAX_THREADS = 256;
 // The approximate 32-bit fixed-point Asian kernels run 4 CTAs per SM (<= 128
 // registers, measured 8-16% faster than their natural ~144), as do the
 // corrections whose natural allocation lies just above.
-// The static FP32 exact kernels need 80-87 registers and are held to 80.
+// The FP32 exact kernels need 80-96 registers and are held to 80 but for three
+// device-scheduled ones; the binary16 / bfloat16 corrections' static launches
+// need up to 104 and are held to 96.
 // Every other instantiation keeps its natural allocation (a cap there spills).
 constexpr int LAUNCH_THREADS = 128;
 template <int EST, int XP, int AP, int SCHEME, int PC, bool DYN = false> struct MinCtas {
   static constexpr bool EM_TERMINAL_FX32 = AP == AP_FX32 && SCHEME == 0 && PC == PC_TERMINAL;
+  static constexpr bool FX = AP == AP_FX32 || AP == AP_FX64;
   static constexpr int value =
-      (EM_TERMINAL_FX32 && (EST == EST_APPROX || (EST == EST_CORR && !DYN))) || (EST == EST_EXACT && XP == XP_F32 && !DYN)
-          ? 6
-      : ((EST == EST_CORR && (AP == AP_FX32 || AP == AP_FX64)) || (EST == EST_APPROX && AP == AP_FX32 && PC == PC_ASIAN)
-             ? 4 : 1);
+      EM_TERMINAL_FX32 && (EST == EST_APPROX || (EST == EST_CORR && !DYN)) ? 6
+      : EST == EST_EXACT && XP == XP_F32 ? (!DYN || (SCHEME == 0 && PC != PC_ASIAN) ? 6 : 1)
+      : EST == EST_CORR && FX ? 4
+      : EST == EST_CORR && AP != AP_FIXED && !DYN ? (SCHEME == 1 && PC == PC_ASIAN ? 4 : 5)
+      : EST == EST_APPROX && AP == AP_FX32 && PC == PC_ASIAN ? 4 : 1;
 };
 
 // The inverse-Normal cubics of the FP32 exact path in shared memory, the same
@@ -120,10 +124,15 @@ __device__ __forceinline__ int32_t ff_sum1(const FastFixed &ff, int32_t z, int32
 // 2's ranks (corrections); chosen once per chunk, so the hot step code has no
 // branch on the method.  FP64 exact kernels: 0 increments in 64-bit integers
 // (exact64.cuh), 1 in FP64.
-// PRE (merged nested kernel, family 24): the 32-bit fast datapath's sum1
-// arrives multiplied by 2^(32 - rs2) (the host proved that it fits), so the
-// rounded product rd(S sum1) is the high word of one 64-bit multiply-add: no
-// funnel shift on the ALU pipe, which bounds that kernel.
+// PRE: the 32-bit fast datapath in its pre-scaled form, for items whose bounds
+// allow it (FastFixed::pre_ok).  sum1 is kept times 2^(32 - rs2), so the rounded
+// product rd(S sum1) is the high word of one 64-bit multiply-add, with no
+// shift; and, mul1 and sum1 having the same grid, sum1 is mul1 plus a constant.
+// Euler: the table holds P_j = con2 Z~_j + radd1 alone (4 bytes): a fine step's
+// mul1 is P_j >> rs1 and a coarse step's (P_j + P_j' - radd1) >> rs1.  The
+// 8-byte pairs' random reads cost 6.2 shared-memory wavefronts a warp, which
+// held shared memory 83% busy in the packed approximate kernel; 4-byte reads
+// cost 3.5.  Milstein: the pairs (Z~_j, scaled sum1_j).
 // MERGED: the merged nested kernel's instantiation, which takes no enumerated
 // items (the plan keeps those apart), so its group code has no enumeration
 // branch.
@@ -146,12 +155,13 @@ struct LevelSim {
   using AS = typename std::conditional<AP == AP_FX32, int32_t, int64_t>::type;  // fixed-point S
   // saturation flag of the fast datapath: OR of (clamped ^ unclamped) for a 32-bit S
   using SatT = typename std::conditional<AP == AP_FX32, uint32_t, bool>::type;
-  // Approximate-only 32-bit datapath: when the host proved it exact (ff.lazy),
-  // a group of packs first runs with S unclamped, tracking only its running
+  // 32-bit datapath: when the host proved it exact (ff.lazy), a group of packs
+  // (or a correction's samples) first runs with S unclamped, tracking only its running
   // maximum hi; if hi stayed at or below lim_S no clamp would have acted and the
   // values are final, otherwise the group runs again on the clamped (EAGER)
   // datapath.
-  static constexpr bool LAZY = (EST == EST_APPROX && AP == AP_FX32);
+  static constexpr bool LAZY = (AP == AP_FX32 && (EST == EST_APPROX || EST == EST_CORR));
+  static constexpr bool P32 = AP == AP_FX32 && PRE && !MIL;   // the table holds P_j only
   static constexpr int KPV = KP;
   static constexpr int ESTV = EST;
   using X = typename XType<XP>::T;
@@ -166,8 +176,11 @@ struct LevelSim {
   // ---- per-item constants (registers) ----
   int level, nsteps, payoff, d, dshift, method;
   // FX32: byte offset of lane l's table entry = rotr(word, rot[l]) & off_mask
-  int32_t pre2;            // PRE: 2^(32 - rs2), and radd2 times it
+  // PRE: 2^(32 - rs2); radd2 times it; what the fine and the coarse step's sum1
+  // add to mul1, times it
+  int32_t pre2, c1p, c1cp;
   int64_t radd2p;
+  static constexpr int LG = P32 ? 2 : 3;   // log2 of a table entry's bytes
   uint32_t rot[KP], off_mask;
   const uint16_t *perm_s;  // method 2 coupling of the exact path (shared memory), or nullptr
   const float4 *phi;       // FP32 exact path: the inverse-Normal cubics in shared memory
@@ -226,6 +239,8 @@ struct LevelSim {
     if constexpr (AP == AP_FX32 && PRE) {
       pre2 = 1 << (32 - it.ff.rs2);
       radd2p = (int64_t)((uint64_t)it.ff.radd2 << (32 - it.ff.rs2));
+      c1p = (int32_t)((uint32_t)(it.ff.con1r >> it.ff.rs_sum1) << (32 - it.ff.rs2));
+      c1cp = (int32_t)((uint32_t)(it.ff.con1cr >> it.ff.rs_sum1) << (32 - it.ff.rs2));
     }
     if constexpr (HALF) {
       hc1 = HO::from_bits(it.h_c1); hc1c = HO::from_bits(it.h_c1c);
@@ -240,10 +255,10 @@ struct LevelSim {
     unit_scale = it.unit_scale;
     smem_tab = tab;
     if constexpr (AP == AP_FX32) {
-      // lane l's field, bits [32 - d(l+1), 32 - d l) of the word, lands at bits [3, 3 + d)
+      // lane l's field, bits [32 - d(l+1), 32 - d l) of the word, lands at bits [LG, LG + d)
 #pragma unroll
-      for (int l = 0; l < KP; ++l) rot[l] = (uint32_t)(32 - it.d * (l + 1) - 3) & 31u;
-      off_mask = ((1u << it.d) - 1u) << 3;
+      for (int l = 0; l < KP; ++l) rot[l] = (uint32_t)(32 - it.d * (l + 1) - LG) & 31u;
+      off_mask = ((1u << it.d) - 1u) << LG;
     }
     perm_s = nullptr;
     if constexpr (HAS_EXACT && XP == XP_F32) {
@@ -341,17 +356,52 @@ struct LevelSim {
   }
   template <bool EAGER>
   __device__ __forceinline__ AS ff_step(AS s, int32_t z, int32_t c1r, int64_t m, SatT &satb) {
-    if constexpr (AP == AP_FX32 && PRE) return ff_apply<EAGER>(s, ff_sum1<MIL, true>(ff, z, c1r, m) * pre2, satb);
-    else return ff_apply<EAGER>(s, ff_sum1<MIL, AP == AP_FX32>(ff, z, c1r, m), satb);
+    return ff_apply<EAGER>(s, ff_sum1<MIL, AP == AP_FX32>(ff, z, c1r, m), satb);
   }
-  // FX32: (Z~, sum1 of a fine step) of lane l of word w, from the shared-memory pairs
-  // (the table sits at the start of the dynamic shared memory: addressing it
+  // FX32: byte offset of lane l's table entry for word w.  Lane 0's field (and
+  // the only one of an unpacked word) is the top one: no mask.
+  __device__ __forceinline__ uint32_t fx32_off(uint32_t w, int l) const {
+    if (l == 0) return (w >> dshift) << LG;
+    return __funnelshift_r(w, w, rot[l]) & off_mask;
+  }
+  // The table sits at the start of the dynamic shared memory: addressing it
   // there, rather than through smem_tab, leaves the base to the load's
-  // immediate offset, one add fewer per lookup)
-  __device__ __forceinline__ int2 fx32_entry(uint32_t w, int l) const {
+  // immediate offset, one add fewer per lookup.
+  template <class E>
+  __device__ __forceinline__ E fx32_entry(uint32_t off) const {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
-    const uint32_t off = __funnelshift_r(w, w, rot[l]) & off_mask;
-    return *(const int2 *)(smem_dyn + off);
+    return *(const E *)(smem_dyn + off);
+  }
+  // The FX32 fine step of lane l on word w; returns what the coarse step needs of
+  // it (Z~, or P_j).  TRACK as in ff_apply.
+  template <bool EAGER, bool TRACK>
+  __device__ __forceinline__ int32_t fx32_fine(uint32_t w, int l) {
+    if constexpr (P32) {
+      const int32_t q = fx32_entry<int32_t>(fx32_off(w, l));
+      aS[l] = ff_apply<EAGER, TRACK>(aS[l], (q >> ff.rs1) * pre2 + c1p, satb[l]);
+      return q;
+    } else {
+      const int2 e = fx32_entry<int2>(fx32_off(w, l));
+      aS[l] = ff_apply<EAGER, TRACK>(aS[l], e.y, satb[l]);
+      return e.x;
+    }
+  }
+  // The FX32 coarse step from the two fine steps' values.
+  template <bool EAGER>
+  __device__ __forceinline__ void fx32_coarse(int l, int32_t x0, int32_t x1) {
+    if constexpr (P32) {
+      const int32_t q = x0 + x1 - (int32_t)ff.radd1;
+      aSc[l] = ff_apply<EAGER>(aSc[l], (q >> ff.rs1) * pre2 + c1cp, satb[l]);
+    } else if constexpr (PRE) {
+      const int32_t z = x0 + x1;
+      const int64_t p1 = (int64_t)ff.con2 * z + ff.radd1;
+      const int64_t p3 = (int64_t)ff.con3 * (z * z - (int32_t)ff.mcoarse) + ff.radd3;
+      const int32_t mul = (int32_t)__funnelshift_r((uint32_t)p1, (uint32_t)((uint64_t)p1 >> 32), ff.rs1) +
+                          (int32_t)__funnelshift_r((uint32_t)p3, (uint32_t)((uint64_t)p3 >> 32), ff.rs3);
+      aSc[l] = ff_apply<EAGER>(aSc[l], mul * pre2 + c1cp, satb[l]);
+    } else {
+      aSc[l] = ff_step<EAGER>(aSc[l], x0 + x1, ff.con1cr, ff.mcoarse, satb[l]);
+    }
   }
 
   // ---- half-precision step (one rounding per operation) ----
@@ -536,20 +586,19 @@ struct LevelSim {
       // its own from Z~_2k + Z~_2k+1
 #pragma unroll
       for (int l = 0; l < KP; ++l) {
-        const int2 e = fx32_entry(J, l);
         if constexpr (PC == PC_ASIAN) { if (i > 0) aaccF[l] += aS[l]; }
         // lazy runs track S after the odd fine steps only (limT); with the parity
         // unknown at compile time, after every step (more is as exact)
         constexpr bool TRACK_FINE = PAR == 1 || (PAR == -1 && COARSE);
-        aS[l] = ff_apply<EAGER, TRACK_FINE>(aS[l], e.y, satb[l]);
+        const int32_t x = fx32_fine<EAGER, TRACK_FINE>(J, l);
         if constexpr (PC == PC_LOOKBACK) aminF[l] = aS[l] < aminF[l] ? aS[l] : aminF[l];
         if constexpr (COARSE) {
           if (odd) {
             if constexpr (PC == PC_ASIAN) { if (i > 1) aaccC[l] += aSc[l]; }
-            aSc[l] = ff_step<EAGER>(aSc[l], azprev[l] + e.x, ff.con1cr, ff.mcoarse, satb[l]);
+            fx32_coarse<EAGER>(l, azprev[l], x);
             if constexpr (PC == PC_LOOKBACK) aminC[l] = aSc[l] < aminC[l] ? aSc[l] : aminC[l];
           } else {
-            azprev[l] = e.x;
+            azprev[l] = x;
           }
         }
       }
@@ -595,9 +644,10 @@ struct LevelSim {
 
   // ---- payoffs ----
   // lg: log2 of the path's steps
+  template <int PAY = -1>
   __device__ __forceinline__ X exact_payoff(X x, X acc, X mn, int lg) const {
     if constexpr (PC == PC_TERMINAL) {
-      if (payoff == 1) return above(x, K) ? X(1) : X(0);
+      if (PAY >= 0 ? PAY == 1 : payoff == 1) return above(x, K) ? X(1) : X(0);
       const X dd = x - K;
       return above(dd, X(0)) ? dd : X(0);
     } else if constexpr (PC == PC_ASIAN) {
@@ -666,8 +716,8 @@ struct LevelSim {
     uint32_t lsat = 0;
     const bool coarse = LV >= 0 ? LV == 1 : level > 0;
     if constexpr (HAS_EXACT) {
-      pf = exact_payoff(S, accF, minF, level);
-      if (coarse) pc = exact_payoff(Sc, accC, minC, level - 1);
+      pf = exact_payoff<PAY>(S, accF, minF, level);
+      if (coarse) pc = exact_payoff<PAY>(Sc, accC, minC, level - 1);
     }
     if constexpr (FIXED) {
       qf = fixed_payoff<PAY>(aS[l], aaccF[l], aminF[l], nsteps, false);
@@ -768,6 +818,12 @@ struct ThreadAcc {
     asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(gsum) : "r"(y), "r"(1));
     asm("mad.wide.s32 %0, %1, %1, %0;" : "+l"(gq) : "r"(y));
   }
+  // two samples, 0 <= y <= 2^30 (payoffs of a 32-bit S): their sum fits 32 bits
+  __device__ __forceinline__ void add_group2(int32_t y0, int32_t y1) {
+    asm("mad.wide.u32 %0, %1, %2, %0;" : "+l"(gsum) : "r"((uint32_t)y0 + (uint32_t)y1), "r"(1));
+    asm("mad.wide.s32 %0, %1, %1, %0;" : "+l"(gq) : "r"(y0));
+    asm("mad.wide.s32 %0, %1, %1, %0;" : "+l"(gq) : "r"(y1));
+  }
   __device__ __forceinline__ void flush_group() {
     isum += gsum;
     add_u128(q_lo, q_hi, gq, 0);
@@ -778,15 +834,17 @@ struct ThreadAcc {
     gsum = 0;
     gq = 0;
   }
-  // Integer sums at the start of a group, to undo the group's samples (the
-  // path-dependent payoffs add each sample to the totals directly).
+  // Sums at the start of a group, to undo the group's samples (the
+  // path-dependent payoffs and the corrections add each sample directly).
   struct Mark {
     int64_t isum;
     uint64_t q_lo, q_hi;
+    float fs, fc, fs2, fc2;
   };
-  __device__ __forceinline__ Mark mark() const { return Mark{isum, q_lo, q_hi}; }
+  __device__ __forceinline__ Mark mark() const { return Mark{isum, q_lo, q_hi, fs, fc, fs2, fc2}; }
   __device__ __forceinline__ void rewind(const Mark &m) {
     isum = m.isum; q_lo = m.q_lo; q_hi = m.q_hi;
+    fs = m.fs; fc = m.fc; fs2 = m.fs2; fc2 = m.fc2;
   }
   // s + y = t + e exactly (Knuth's TwoSum, six FP32 operations): s becomes t, e is returned.
   static __device__ __forceinline__ float two_sum(float &s, float y) {
@@ -894,6 +952,10 @@ struct GroupCtx {
   int d, level, enumerate, lanes;
   uint64_t first, last;
 };
+// The Philox words of call q.
+__device__ __forceinline__ uint4 draw(const GroupCtx &it, const LaunchArgs &args, uint64_t q) {
+  return philox4x32_10(make_uint4((uint32_t)q, (uint32_t)(q >> 32), it.ctr2, it.ctr3), args.rk);
+}
 
 // The samples of group g of a chunk, for a level class LC known at compile
 // time (0: level 0, 1: level 1, 2: levels >= 2).  A group is one Philox call's
@@ -920,16 +982,19 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
     uint64_t qbase = P * calls;
     if constexpr (E && Sim::LAZY) opaque(qbase);
     sim.begin();
-    // qbase is a multiple of calls (a power of two): the calls share its high word
+    // qbase is a multiple of calls (a power of two): the calls share its high
+    // word (packed draws, whose calls feed three samples, keep the registers)
     const PhiloxStream ps((uint32_t)(qbase >> 32), it.ctr2, it.ctr3, args.rk);
     for (uint32_t c = 0; c < calls; ++c) {
-      const uint4 w = ps.call((uint32_t)qbase + c, args.rk);
+      const uint4 w = KP == 1 ? ps.call((uint32_t)qbase + c, args.rk) : draw(it, args, qbase + c);
       const int i0 = (int)(c << 2);
       sim.template step<true, 0, E>(w.x << lsh, i0);
       sim.template step<true, 1, E>(w.y << lsh, i0 + 1);
       sim.template step<true, 0, E>(w.z << lsh, i0 + 2);
       sim.template step<true, 1, E>(w.w << lsh, i0 + 3);
     }
+    // a lazy correction that left its range adds nothing and runs again
+    if (Sim::ESTV == EST_CORR && !E && sim.over()) return;
 #pragma unroll
     for (int l = 0; l < KP; ++l) {
       const uint64_t s = KP == 1 ? g : P * KP + l;
@@ -940,11 +1005,8 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
     uint64_t gw = g;
     if constexpr (E && Sim::LAZY) opaque(gw);
     uint4 w;
-    if constexpr (Sim::ENUMERATE)
-      w = it.enumerate ? enum_words(gw, LC, it.d)
-                       : philox4x32_10(make_uint4((uint32_t)gw, (uint32_t)(gw >> 32), it.ctr2, it.ctr3), args.rk);
-    else
-      w = philox4x32_10(make_uint4((uint32_t)gw, (uint32_t)(gw >> 32), it.ctr2, it.ctr3), args.rk);
+    if (Sim::ENUMERATE && it.enumerate) w = enum_words(gw, LC, it.d);
+    else w = draw(it, args, gw);
     constexpr int PPG = LC == 1 ? 2 : 4;  // packs per group
     const uint64_t s0 = (uint64_t)(PPG * KP) * g;
     // samples s0 + k are valid for k in [klo, khi)
@@ -988,15 +1050,18 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
 template <bool FULL, class Sim, class Acc>
 __device__ __forceinline__ void y0_group(const Sim &sim, Acc &acc, const uint4 &w, int klo, int khi) {
   constexpr int KP = Sim::KPV;
+  int32_t y[4 * KP];
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
 #pragma unroll
     for (int l = 0; l < KP; ++l) {
       const int k = u * KP + l;
-      const int32_t y = sim.fx32_entry(word_of(w, u), l).x;
-      acc.add_group(FULL || (k >= klo && k < khi) ? y : 0);
+      y[k] = sim.template fx32_entry<int32_t>(sim.fx32_off(word_of(w, u), l) >> (Sim::LG - 2));
+      if (!(FULL || (k >= klo && k < khi))) y[k] = 0;
     }
   }
+#pragma unroll
+  for (int k = 0; k < 4 * KP; k += 2) acc.add_group2(y[k], y[k + 1]);
   acc.flush_group();
 }
 
@@ -1010,11 +1075,8 @@ __device__ __forceinline__ void group_loop_y0(const Sim &sim, Acc &acc, const La
   for (uint32_t r = threadIdx.x; r < ng; r += blockDim.x) {
     const uint64_t g = gbeg + r;
     uint4 w;
-    if constexpr (Sim::ENUMERATE)
-      w = it.enumerate ? enum_words(g, 0, it.d)
-                       : philox4x32_10(make_uint4((uint32_t)g, (uint32_t)(g >> 32), it.ctr2, it.ctr3), args.rk);
-    else
-      w = philox4x32_10(make_uint4((uint32_t)g, (uint32_t)(g >> 32), it.ctr2, it.ctr3), args.rk);
+    if (Sim::ENUMERATE && it.enumerate) w = enum_words(g, 0, it.d);
+    else w = draw(it, args, g);
     if (r >= rf0 && r < rf1) {
       y0_group<true>(sim, acc, w, 0, 0);
     } else {
@@ -1048,7 +1110,15 @@ __device__ __forceinline__ void group_loop(Sim &sim, ThreadAcc<EST, XP> &acc, co
     const bool full = r >= rf0 && r < rf1;
     if constexpr (Sim::LAZY && !DUMP) {
       bool eager = true;
-      if (lazy && full) {
+      if constexpr (EST == EST_CORR) {
+        if (lazy) {
+          sim.hi = 0;
+          const auto saved = acc.mark();
+          run_group<LC, false, false, PAYF, DUMP>(sim, acc, args, it, g, full, first, last, dump);
+          eager = sim.over();
+          if (LC != 2 && eager) acc.rewind(saved);
+        }
+      } else if (lazy && full) {
         sim.hi = 0;
         if constexpr (PC == PC_TERMINAL) {
           // the group's sums stay in their own accumulator until the group is kept
@@ -1110,9 +1180,7 @@ __device__ __forceinline__ void chunk_body(const LaunchArgs &args, const ItemDes
   mlmc_sample_rec *dump = DUMP ? (mlmc_sample_rec *)it.dump : nullptr;
   const bool lazy = Sim::LAZY && !DUMP && it.ff.lazy;
   const int lc = it.level >= 2 ? 2 : it.level;
-  GroupCtx gx;
-  gx.ctr2 = it.ctr2; gx.ctr3 = it.ctr3; gx.d = it.d; gx.level = it.level; gx.enumerate = it.enumerate;
-  gx.lanes = it.lanes; gx.first = it.first; gx.last = it.first + it.N;
+  const GroupCtx gx{it.ctr2, it.ctr3, it.d, it.level, it.enumerate, it.lanes, it.first, it.first + it.N};
   auto loop = [&](auto lctag, auto paytag) {
     group_loop<decltype(lctag)::value, decltype(paytag)::value, DUMP, EST, XP, AP, PC>(sim, acc, args, gx, gbeg, ng,
                                                                                       rf0, rf1, lazy, dump);
@@ -1122,8 +1190,11 @@ __device__ __forceinline__ void chunk_body(const LaunchArgs &args, const ItemDes
   using L2 = std::integral_constant<int, 2>;
   if constexpr (Sim::LAZY && !DUMP && PC == PC_TERMINAL) {
     const bool dig = it.payoff == 1;
+    const bool y0 = EST == EST_APPROX && it.tab_y0;
     if (lc == 0) {
-      if (it.tab_y0) group_loop_y0(sim, acc, args, gx, gbeg, ng, rf0, rf1);
+      if (y0) {
+        if constexpr (EST == EST_APPROX) group_loop_y0(sim, acc, args, gx, gbeg, ng, rf0, rf1);
+      }
       else if (dig) loop(L0{}, PayTag<1>{});
       else loop(L0{}, PayTag<0>{});
     }
@@ -1168,11 +1239,15 @@ __device__ __forceinline__ void chunk_body(const LaunchArgs &args, const ItemDes
   }
 }
 
+// Does an item run the pre-scaled form of the 32-bit fast datapath?  (Records
+// take the plain form, as does Method 2's coupled exact path: pre_ok is 0 there.)
+__device__ __forceinline__ bool fx32_pre(const ItemDesc &it) { return it.ff.pre_ok && !it.dump; }
+
 // Find the item of chunk gc (the last with chunk_begin <= gc) and stage its
 // approximate-Normal table in shared memory (unless *staged, when given, says
 // that it is there already).  Every thread has finished the previous chunk
 // before the table is overwritten (block_reduce_write ends with a barrier).
-template <int AP, int SCHEME, bool PRE = false, bool PHI_BY_KIND = false>
+template <int AP, int SCHEME, bool PHI_BY_KIND = false>
 __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, uint32_t gc, const void **staged) {
   extern __shared__ __align__(16) unsigned char smem_tab[];
   __shared__ int s_item;
@@ -1199,9 +1274,11 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
   const int item = s_item;
   const ItemDesc &it = items[item];
   if constexpr (AP == AP_FX32) {
-    // (Z~_j, sum1 of a fine step from Z~_j) for every index j: Method 1 and 2
-    // values from the item's table, Method 3 values from its class lines (the
-    // arithmetic of LevelSim::fixed_z); sum1 by the datapath's own step code.
+    // (Z~_j, sum1 of a fine step from Z~_j) for every index j, or in the
+    // pre-scaled form of Euler items P_j = con2 Z~_j + radd1 (LevelSim's PRE):
+    // Method 1 and 2 values from the item's table, Method 3 values from its
+    // class lines (the arithmetic of LevelSim::fixed_z); sum1 by the datapath's
+    // own step code.
     // The table depends on the item's constants as well, so a persistent CTA
     // (staged != nullptr) keeps it while its chunks stay in the same item.
     if (staged && *staged == (const void *)&it) return item;
@@ -1218,7 +1295,9 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
     // merged launch: only the correction chunks (kind 2) run the FP32 exact path;
     // the copies proceed while the pairs are formed
     if (PHI_BY_KIND && it.kind == 2) stage_phi_inv(phi_inv_smem());
+    const bool pre = fx32_pre(it), p32 = pre && SCHEME == 0;
     int2 *dst = (int2 *)smem_tab;
+    int32_t *dst4 = (int32_t *)smem_tab;
     const M3Coef *m3 = (const M3Coef *)ztab;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
       int32_t z;
@@ -1231,6 +1310,10 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
         const int sh = M3_FRAC - fZh;
         const int32_t v = (int32_t)((t + ((int64_t)1 << (sh - 1))) >> sh);
         z = ai.neg ? -v : v;
+      }
+      if (p32 && !tab_y0) {
+        dst4[k] = ff.con2 * z + (int32_t)ff.radd1;
+        continue;
       }
       const int32_t sum1 = ff_sum1<SCHEME == 1, true>(ff, z, ff.con1r, ff.mfine);
       if (tab_y0) {
@@ -1247,9 +1330,9 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
         const int32_t lim = (int32_t)ff.limS;
         const int32_t c = min(max(s1, -lim), lim);
         const int32_t y = c > Kq ? (payoff == 1 ? (int32_t)1 << fS : c - Kq) : 0;
-        dst[k] = make_int2(y, c != s1 ? 1 : 0);
+        dst4[k] = y;
       } else {
-        dst[k] = make_int2(z, PRE ? sum1 * (1 << (32 - ff.rs2)) : sum1);
+        dst[k] = make_int2(z, pre ? sum1 * (1 << (32 - ff.rs2)) : sum1);
       }
     }
     if (it.perm) {   // after the table: the method-2 interval ranks
@@ -1286,6 +1369,18 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
   return item;
 }
 
+// A chunk of the 32-bit fast datapath in the form that its item takes.
+template <int EST, int SCHEME, int PC, int KP, bool DYN, bool MERGED>
+__device__ __forceinline__ void fx32_chunk(const LaunchArgs &args, const ItemDesc &it, int item, uint32_t gc,
+                                           const unsigned char *smem_tab) {
+  if (fx32_pre(it))
+    chunk_body<EST, XP_F32, AP_FX32, SCHEME, PC, KP, 0, false, DYN, true, MERGED>(args, it, item, gc, smem_tab);
+  else if (EST != EST_CORR || !it.perm)
+    chunk_body<EST, XP_F32, AP_FX32, SCHEME, PC, KP, 0, false, DYN, false, MERGED>(args, it, item, gc, smem_tab);
+  else if constexpr (EST == EST_CORR)
+    chunk_body<EST, XP_F32, AP_FX32, SCHEME, PC, KP, 4, false, DYN, false, MERGED>(args, it, item, gc, smem_tab);
+}
+
 // One chunk (gc) of one launch: its item and table (stage_chunk), then the
 // chunk's sample groups and the CTA's Partial for the chunk.
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP, bool ALLOW_DUMP, bool DYN>
@@ -1299,13 +1394,11 @@ __device__ __forceinline__ void run_chunk(const LaunchArgs &args, const ItemDesc
   } else if constexpr (XP == XP_F64) {
     if (it.qF) chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
     else chunk_body<EST, XP, AP, SCHEME, PC, KP, 1, false, DYN>(args, it, item, gc, smem_tab);
-  } else if constexpr (AP == AP_NONE || AP == AP_FX32) {
-    // no method choice: exact paths, and the FX32 table that holds every method's values
-    if (EST == EST_CORR && it.perm) {
-      if constexpr (EST == EST_CORR) chunk_body<EST, XP, AP, SCHEME, PC, KP, 4, false, DYN>(args, it, item, gc, smem_tab);
-    } else {
-      chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
-    }
+  } else if constexpr (AP == AP_NONE) {
+    chunk_body<EST, XP, AP, SCHEME, PC, KP, 0, false, DYN>(args, it, item, gc, smem_tab);
+  } else if constexpr (AP == AP_FX32) {
+    // no method choice: the table holds every method's values
+    fx32_chunk<EST, SCHEME, PC, KP, DYN, false>(args, it, item, gc, smem_tab);
   } else {
     if (EST == EST_CORR && it.perm) {
       if constexpr (EST == EST_CORR) chunk_body<EST, XP, AP, SCHEME, PC, KP, 4, false, DYN>(args, it, item, gc, smem_tab);
@@ -1354,21 +1447,25 @@ level_kernel_dyn(const __grid_constant__ LaunchArgs args) {
 // Its chunks run the same chunk bodies as the separate launches, in one grid
 // ordered by decreasing CTA cost, so the longest chains start first and the
 // short chunks of every family fill in behind them.
-// PRE: every item's sum1 fits the pre-scaled product (family 24; see LevelSim).
-template <int AP, int SCHEME, int PC, bool PRE>
+// PRE: every item takes the pre-scaled form (family 24; else family 17).
+template <int SCHEME, int PC, bool PRE>
 __global__ void __launch_bounds__(LAUNCH_THREADS, 6) nested_kernel(const __grid_constant__ LaunchArgs args) {
   extern __shared__ __align__(16) unsigned char smem_tab[];
   const uint32_t gc = args.chunk0 + blockIdx.x;
-  const int item = stage_chunk<AP, SCHEME, PRE, true>(args.items, args.n_items, gc, nullptr);
+  const int item = stage_chunk<AP_FX32, SCHEME, true>(args.items, args.n_items, gc, nullptr);
   const ItemDesc &it = args.items[item];
-  if (it.kind == 0)
-    chunk_body<EST_APPROX, XP_F32, AP, SCHEME, PC, 3, 0, false, false, PRE, true>(args, it, item, gc, smem_tab);
-  else if (it.kind == 1)
-    chunk_body<EST_APPROX, XP_F32, AP, SCHEME, PC, 1, 0, false, false, PRE, true>(args, it, item, gc, smem_tab);
-  else if (it.perm)
-    chunk_body<EST_CORR, XP_F32, AP, SCHEME, PC, 1, 4, false, false, PRE, true>(args, it, item, gc, smem_tab);
-  else
-    chunk_body<EST_CORR, XP_F32, AP, SCHEME, PC, 1, 0, false, false, PRE, true>(args, it, item, gc, smem_tab);
+  if constexpr (PRE) {
+    if (it.kind == 0)
+      chunk_body<EST_APPROX, XP_F32, AP_FX32, SCHEME, PC, 3, 0, false, false, true, true>(args, it, item, gc, smem_tab);
+    else if (it.kind == 1)
+      chunk_body<EST_APPROX, XP_F32, AP_FX32, SCHEME, PC, 1, 0, false, false, true, true>(args, it, item, gc, smem_tab);
+    else
+      chunk_body<EST_CORR, XP_F32, AP_FX32, SCHEME, PC, 1, 0, false, false, true, true>(args, it, item, gc, smem_tab);
+  } else {
+    if (it.kind == 0) fx32_chunk<EST_APPROX, SCHEME, PC, 3, false, true>(args, it, item, gc, smem_tab);
+    else if (it.kind == 1) fx32_chunk<EST_APPROX, SCHEME, PC, 1, false, true>(args, it, item, gc, smem_tab);
+    else fx32_chunk<EST_CORR, SCHEME, PC, 1, false, true>(args, it, item, gc, smem_tab);
+  }
 }
 
 }  // namespace mlmc
