@@ -55,10 +55,11 @@ constexpr int MAX_THREADS = 256;
 // corrections whose natural allocation lies just above.
 // The FP32 exact kernels need 80-96 registers and are held to 80 but for three
 // device-scheduled ones; the binary16 / bfloat16 corrections' static launches
-// need up to 104 and are held to 96.
+// need up to 104 and are held to 96, and the unpacked binary16 / bfloat16
+// approximate kernels' (two samples per thread from level 2), 84-96, to 80.
 // Every other instantiation keeps its natural allocation (a cap there spills).
 constexpr int LAUNCH_THREADS = 128;
-template <int EST, int XP, int AP, int SCHEME, int PC, bool DYN = false> struct MinCtas {
+template <int EST, int XP, int AP, int SCHEME, int PC, int KP, bool DYN = false> struct MinCtas {
   static constexpr bool EM_TERMINAL_FX32 = AP == AP_FX32 && SCHEME == 0 && PC == PC_TERMINAL;
   static constexpr bool FX = AP == AP_FX32 || AP == AP_FX64;
   static constexpr int value =
@@ -66,7 +67,8 @@ template <int EST, int XP, int AP, int SCHEME, int PC, bool DYN = false> struct 
       : EST == EST_EXACT && XP == XP_F32 ? (!DYN || (SCHEME == 0 && PC != PC_ASIAN) ? 6 : 1)
       : EST == EST_CORR && FX ? 4
       : EST == EST_CORR && AP != AP_FIXED && !DYN ? (SCHEME == 1 && PC == PC_ASIAN ? 4 : 5)
-      : EST == EST_APPROX && AP == AP_FX32 && PC == PC_ASIAN ? 4 : 1;
+      : EST == EST_APPROX && AP == AP_FX32 && PC == PC_ASIAN ? 4
+      : EST == EST_APPROX && KP == 1 && !DYN && AP != AP_FIXED && !FX ? 6 : 1;
 };
 
 // The inverse-Normal cubics of the FP32 exact path in shared memory, the same
@@ -150,8 +152,12 @@ struct LevelSim {
   static constexpr bool HALF = (AP == AP_F16 || AP == AP_BF16 || AP == AP_F16S || AP == AP_BF16S);
   // half increments with S (and its average and minimum) in FP32
   static constexpr bool S32 = (AP == AP_F16S || AP == AP_BF16S);
-  // packed half draws: lanes 0 and 1 share paired (x2) registers, lane 2 is scalar
-  static constexpr bool PAIR = HALF && KP == 3 && !S32;
+  // Half arithmetic on two lanes at once, in paired (x2) registers: lanes 0 and 1
+  // of packed draws (lane 2 is scalar), or two samples of one thread with words
+  // of their own (DUO, KP = 2).  The half instructions run on the pipe of the
+  // integer multiplies, at its rate whether they hold one value or two.
+  static constexpr bool DUO = HALF && KP == 2;
+  static constexpr bool PAIR = HALF && KP >= 2 && !S32;
   using AS = typename std::conditional<AP == AP_FX32, int32_t, int64_t>::type;  // fixed-point S
   // saturation flag of the fast datapath: OR of (clamped ^ unclamped) for a 32-bit S
   using SatT = typename std::conditional<AP == AP_FX32, uint32_t, bool>::type;
@@ -248,7 +254,7 @@ struct LevelSim {
       if constexpr (S32) hS0 = it.S0f;
       else hS0 = HO::from_bits(it.h_S0);
       K32 = it.Kf;
-      if constexpr (PAIR) {
+      if constexpr (PAIR || DUO) {
         pc1 = HO2::splat(hc1); pc1c = HO2::splat(hc1c); pc2 = HO2::splat(hc2); pc3 = HO2::splat(hc3);
       }
     }
@@ -290,8 +296,9 @@ struct LevelSim {
       sat[l] = 0;
     }
     if constexpr (PAIR) {
-      pS = HO2::splat(hS0); pSc = pS; pzprev = HO2::splat(HO::from_f(0.0f));
+      pS = HO2::splat(hS0); pSc = pS;
     }
+    if constexpr (PAIR || DUO) pzprev = HO2::splat(HO::from_f(0.0f));
   }
   // LAZY: did some S since hi was reset leave [-lim_S, lim_S]?  (The host
   // proved that it cannot leave below first.)
@@ -423,8 +430,8 @@ struct LevelSim {
       return HO::add(s, mul2);
     }
   }
-  // the same step on two lanes at once
-  __device__ __forceinline__ H2 h2_step(H2 s, H2 z, H2 cc1, H2 mh) const {
+  // the same on two lanes at once: the increment, and the step
+  __device__ __forceinline__ H2 h2_inc(H2 z, H2 cc1, H2 mh) const {
     const H2 mul1 = HO2::mul(pc2, z);
     H2 sum1 = HO2::add(cc1, mul1);
     if constexpr (MIL) {
@@ -433,8 +440,10 @@ struct LevelSim {
       const H2 mul3 = HO2::mul(pc3, sqm);
       sum1 = HO2::add(sum1, mul3);
     }
-    const H2 mul2 = HO2::mul(s, sum1);
-    return HO2::add(s, mul2);
+    return sum1;
+  }
+  __device__ __forceinline__ H2 h2_step(H2 s, H2 z, H2 cc1, H2 mh) const {
+    return HO2::add(s, HO2::mul(s, h2_inc(z, cc1, mh)));
   }
   // lane l's half state (fine / coarse)
   __device__ __forceinline__ HS lane_S(int l) const {
@@ -483,8 +492,9 @@ struct LevelSim {
 
   // One fine step i driven by J, and the coarse step after odd i (levels >= 1).
   // PAR: parity of i when known at compile time (0 even, 1 odd), -1 otherwise.
+  // J1: the second sample's word (DUO).
   template <bool COARSE, int PAR = -1, bool EAGER = true>
-  __device__ __forceinline__ void step(uint32_t J, int i) {
+  __device__ __forceinline__ void step(uint32_t J, int i, uint32_t J1 = 0) {
     const bool odd = PAR >= 0 ? (PAR == 1) : ((i & 1) != 0);
     if constexpr (HAS_EXACT) {
       // Method 2 (Sec. 3.2): the exact path takes the uniform in the interval
@@ -546,39 +556,71 @@ struct LevelSim {
     }
     if constexpr (PAIR) {
       // Algorithm-1 arithmetic of lanes 0 and 1 in paired instructions; lane 2 alone
-      const H z0 = half_z(J), z1 = half_z(J << d), z2 = half_z(J << (2 * d));
-      const H2 z01 = HO2::pack(z0, z1);
+      constexpr bool THIRD = KP == 3;
+      const H2 z01 = HO2::pack(half_z(J), half_z(DUO ? J1 : J << d));
+      H z2 = HO::from_f(0.0f);
+      if constexpr (THIRD) z2 = half_z(J << (2 * d));
       if constexpr (PC == PC_ASIAN) {
         if (i > 0) {
           haccF[0] = __fadd_rn(haccF[0], HO::to_f(HO2::lo(pS)));
           haccF[1] = __fadd_rn(haccF[1], HO::to_f(HO2::hi(pS)));
-          haccF[2] = __fadd_rn(haccF[2], HO::to_f(hS[2]));
+          if constexpr (THIRD) haccF[2] = __fadd_rn(haccF[2], HO::to_f(hS[2]));
         }
       }
       pS = h2_step(pS, z01, pc1, HO2::splat(HO::from_f(1.0f)));
-      hS[2] = h_step(hS[2], z2, hc1, HO::from_f(1.0f));
+      if constexpr (THIRD) hS[2] = h_step(hS[2], z2, hc1, HO::from_f(1.0f));
       if constexpr (PC == PC_LOOKBACK) {
-        lane_min(hminF[0], HO2::lo(pS)); lane_min(hminF[1], HO2::hi(pS)); lane_min(hminF[2], hS[2]);
+        lane_min(hminF[0], HO2::lo(pS)); lane_min(hminF[1], HO2::hi(pS));
+        if constexpr (THIRD) lane_min(hminF[2], hS[2]);
       }
       if constexpr (COARSE) {
         if (odd) {
           const H2 zc01 = HO2::add(pzprev, z01);
-          const H zc2 = HO::add(hzprev[2], z2);
           if constexpr (PC == PC_ASIAN) {
             if (i > 1) {
               haccC[0] = __fadd_rn(haccC[0], HO::to_f(HO2::lo(pSc)));
               haccC[1] = __fadd_rn(haccC[1], HO::to_f(HO2::hi(pSc)));
-              haccC[2] = __fadd_rn(haccC[2], HO::to_f(hSc[2]));
+              if constexpr (THIRD) haccC[2] = __fadd_rn(haccC[2], HO::to_f(hSc[2]));
             }
           }
           pSc = h2_step(pSc, zc01, pc1c, HO2::splat(HO::from_f(2.0f)));
-          hSc[2] = h_step(hSc[2], zc2, hc1c, HO::from_f(2.0f));
+          if constexpr (THIRD) hSc[2] = h_step(hSc[2], HO::add(hzprev[2], z2), hc1c, HO::from_f(2.0f));
           if constexpr (PC == PC_LOOKBACK) {
-            lane_min(hminC[0], HO2::lo(pSc)); lane_min(hminC[1], HO2::hi(pSc)); lane_min(hminC[2], hSc[2]);
+            lane_min(hminC[0], HO2::lo(pSc)); lane_min(hminC[1], HO2::hi(pSc));
+            if constexpr (THIRD) lane_min(hminC[2], hSc[2]);
           }
         } else {
           pzprev = z01;
-          hzprev[2] = z2;
+          if constexpr (THIRD) hzprev[2] = z2;
+        }
+      }
+    } else if constexpr (DUO) {
+      // the increments of both samples in paired instructions, their FP32 S apart
+      auto apply = [&](HS *s, H2 inc) {
+        s[0] = __fadd_rn(s[0], __fmul_rn(s[0], HO::to_f(HO2::lo(inc))));
+        s[1] = __fadd_rn(s[1], __fmul_rn(s[1], HO::to_f(HO2::hi(inc))));
+      };
+      const H2 z01 = HO2::pack(half_z(J), half_z(J1));
+      if constexpr (PC == PC_ASIAN) {
+        if (i > 0) {
+          haccF[0] = __fadd_rn(haccF[0], sf(hS[0]));
+          haccF[1] = __fadd_rn(haccF[1], sf(hS[1]));
+        }
+      }
+      apply(hS, h2_inc(z01, pc1, HO2::splat(HO::from_f(1.0f))));
+      if constexpr (PC == PC_LOOKBACK) { lane_min(hminF[0], hS[0]); lane_min(hminF[1], hS[1]); }
+      if constexpr (COARSE) {
+        if (odd) {
+          if constexpr (PC == PC_ASIAN) {
+            if (i > 1) {
+              haccC[0] = __fadd_rn(haccC[0], sf(hSc[0]));
+              haccC[1] = __fadd_rn(haccC[1], sf(hSc[1]));
+            }
+          }
+          apply(hSc, h2_inc(HO2::add(pzprev, z01), pc1c, HO2::splat(HO::from_f(2.0f))));
+          if constexpr (PC == PC_LOOKBACK) { lane_min(hminC[0], hSc[0]); lane_min(hminC[1], hSc[1]); }
+        } else {
+          pzprev = z01;
         }
       }
     } else if constexpr (AP == AP_FX32) {
@@ -1151,6 +1193,33 @@ __device__ __forceinline__ void group_loop(Sim &sim, ThreadAcc<EST, XP> &acc, co
   acc.flush_real();
 }
 
+// The first ng groups of a chunk, a multiple of 2 blockDim.x, two at a time
+// (Sim::DUO; levels >= 2, one sample per group): groups r and r + blockDim.x.
+// The binary16 kernel's integer-multiply pipe was 87% busy, half of it with
+// scalar half instructions: 1,000,003 level-8 Milstein Asian samples 386 -> 276 us
+// (with the larger chunks that give a thread two samples there).
+template <class Sim, class Acc>
+__device__ __forceinline__ void group_loop_duo(Sim &sim, Acc &acc, const LaunchArgs &args, const GroupCtx &it,
+                                               uint64_t gbeg, uint32_t ng) {
+  const uint32_t calls = 1u << (it.level - 2);
+  for (uint32_t r = threadIdx.x; r < ng; r += 2u * blockDim.x) {
+    const uint64_t q0 = (gbeg + r) * calls, q1 = q0 + (uint64_t)blockDim.x * calls;
+    const PhiloxStream p0((uint32_t)(q0 >> 32), it.ctr2, it.ctr3, args.rk);
+    const PhiloxStream p1((uint32_t)(q1 >> 32), it.ctr2, it.ctr3, args.rk);
+    sim.begin();
+    for (uint32_t c = 0; c < calls; ++c) {
+      const uint4 w = p0.call((uint32_t)q0 + c, args.rk), v = p1.call((uint32_t)q1 + c, args.rk);
+      const int i0 = (int)(c << 2);
+      sim.template step<true, 0>(w.x, i0, v.x);
+      sim.template step<true, 1>(w.y, i0 + 1, v.y);
+      sim.template step<true, 0>(w.z, i0 + 2, v.z);
+      sim.template step<true, 1>(w.w, i0 + 3, v.w);
+    }
+    sim.template finish<true, -1, 1>(acc, 0, true, nullptr);
+    sim.template finish<true, -1, 1>(acc, 1, true, nullptr);
+  }
+}
+
 // Simulate one chunk of an item (its table already in shared memory) and
 // write the CTA's Partial for it.  The level class and (on the lazy terminal
 // path) the payoff are fixed once per chunk, so the group loop carries no
@@ -1162,25 +1231,41 @@ template <int EST, int XP, int AP, int SCHEME, int PC, int KP, int MSEL, bool DU
 __device__ __forceinline__ void chunk_body(const LaunchArgs &args, const ItemDesc &it, int item, uint32_t gc,
                                            const unsigned char *smem_tab) {
   using Sim = LevelSim<EST, XP, AP, SCHEME, PC, KP, MSEL, PRE, MERGED>;
-  Sim sim;
-  sim.load(it, smem_tab);
+  // unpacked half-precision estimators take a thread's samples two at a time from
+  // level 2 (a thread with one sample, or its odd last one, takes it alone; the
+  // device-scheduled kernels, whose registers it would raise, always do)
+  constexpr bool DUO = EST == EST_APPROX && Sim::HALF && KP == 1 && !DUMP && !DYN;
   ThreadAcc<EST, XP> acc;
   acc.init();
 
   const uint32_t chunk = gc - it.chunk_begin;
   const uint64_t per_chunk = (uint64_t)it.groups_per_thread * blockDim.x;
-  const uint64_t gbeg = it.g0 + (uint64_t)chunk * per_chunk;
+  uint64_t gbeg = it.g0 + (uint64_t)chunk * per_chunk;
   const uint64_t gend = min(it.g1, gbeg + per_chunk);
-  const uint32_t ng = gend > gbeg ? (uint32_t)(gend - gbeg) : 0u;
+  uint32_t ng = gend > gbeg ? (uint32_t)(gend - gbeg) : 0u;
   // the chunk's groups [rf0, rf1) (relative to gbeg) lie entirely in the item's range
   const uint64_t gf0 = max(it.gf0, gbeg), gf1 = min(it.gf1, gend);
-  const uint32_t rf0 = gf0 < gf1 ? (uint32_t)(gf0 - gbeg) : 0u;
-  const uint32_t rf1 = gf0 < gf1 ? (uint32_t)(gf1 - gbeg) : 0u;
+  uint32_t rf0 = gf0 < gf1 ? (uint32_t)(gf0 - gbeg) : 0u;
+  uint32_t rf1 = gf0 < gf1 ? (uint32_t)(gf1 - gbeg) : 0u;
   // per-sample records only in the DUMP instantiation (parity runs)
   mlmc_sample_rec *dump = DUMP ? (mlmc_sample_rec *)it.dump : nullptr;
   const bool lazy = Sim::LAZY && !DUMP && it.ff.lazy;
   const int lc = it.level >= 2 ? 2 : it.level;
   const GroupCtx gx{it.ctr2, it.ctr3, it.d, it.level, it.enumerate, it.lanes, it.first, it.first + it.N};
+  if constexpr (DUO) {
+    const uint32_t pairs = it.level >= 2 && it.lanes <= 1 ? ng / (2u * blockDim.x) * (2u * blockDim.x) : 0u;
+    if (pairs) {
+      LevelSim<EST, XP, AP, SCHEME, PC, 2, MSEL> duo;
+      duo.load(it, smem_tab);
+      group_loop_duo(duo, acc, args, gx, gbeg, pairs);
+      gbeg += pairs;
+      ng -= pairs;
+      rf0 = rf0 > pairs ? rf0 - pairs : 0u;
+      rf1 = rf1 > pairs ? rf1 - pairs : 0u;
+    }
+  }
+  Sim sim;
+  sim.load(it, smem_tab);
   auto loop = [&](auto lctag, auto paytag) {
     group_loop<decltype(lctag)::value, decltype(paytag)::value, DUMP, EST, XP, AP, PC>(sim, acc, args, gx, gbeg, ng,
                                                                                       rf0, rf1, lazy, dump);
@@ -1409,7 +1494,7 @@ __device__ __forceinline__ void run_chunk(const LaunchArgs &args, const ItemDesc
 
 // Static launch: CTA b runs chunk chunk0 + b of the launch.
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
-__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC>::value)
+__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC, KP>::value)
 level_kernel(const __grid_constant__ LaunchArgs args) {
   stage_exact_table<EST, XP>();
   run_chunk<EST, XP, AP, SCHEME, PC, KP, false, false>(args, args.items, args.n_items, args.chunk0 + blockIdx.x,
@@ -1420,7 +1505,7 @@ level_kernel(const __grid_constant__ LaunchArgs args) {
 // its own, so that the record-writing code does not weigh on the register
 // allocation of the launches without records.
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
-__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC>::value)
+__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC, KP>::value)
 level_kernel_dump(const __grid_constant__ LaunchArgs args) {
   stage_exact_table<EST, XP>();
   run_chunk<EST, XP, AP, SCHEME, PC, KP, true, false>(args, args.items, args.n_items, args.chunk0 + blockIdx.x,
@@ -1431,7 +1516,7 @@ level_kernel_dump(const __grid_constant__ LaunchArgs args) {
 // and chunk counts come from args.dyn, written on the device before the
 // launch; CTA b runs chunks b, b + gridDim.x, ...
 template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
-__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC, true>::value)
+__global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC, KP, true>::value)
 level_kernel_dyn(const __grid_constant__ LaunchArgs args) {
   const DynLaunch d = *args.dyn;
   const void *staged = nullptr;
