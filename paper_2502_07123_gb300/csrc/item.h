@@ -154,6 +154,10 @@ struct LaunchArgs {
   // nonzero: some item of the launch writes per-sample records (the launch
   // uses the kernel that holds the record-writing code)
   int dump;
+  // nonzero: the launch's one item is `one`, part of the kernel's own arguments
+  // (a synchronous single-item call then queues no copy before its kernel)
+  int use_one;
+  ItemDesc one;
 };
 
 #if defined(__CUDACC__)

@@ -1336,7 +1336,9 @@ template <int AP, int SCHEME, bool PHI_BY_KIND = false>
 __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, uint32_t gc, const void **staged) {
   extern __shared__ __align__(16) unsigned char smem_tab[];
   __shared__ int s_item;
-  if (threadIdx.x < 32) {
+  if (n_items == 1) {
+    if (threadIdx.x == 0) s_item = 0;
+  } else if (threadIdx.x < 32) {
     // last item with chunk_begin <= gc (chunk_begin is non-decreasing and
     // items[0].chunk_begin <= gc): warp 0 samples 32 evenly spaced items per
     // round, one load each, and narrows to the stride after the last sample
@@ -1497,8 +1499,8 @@ template <int EST, int XP, int AP, int SCHEME, int PC, int KP>
 __global__ void __launch_bounds__(LAUNCH_THREADS, MinCtas<EST, XP, AP, SCHEME, PC, KP>::value)
 level_kernel(const __grid_constant__ LaunchArgs args) {
   stage_exact_table<EST, XP>();
-  run_chunk<EST, XP, AP, SCHEME, PC, KP, false, false>(args, args.items, args.n_items, args.chunk0 + blockIdx.x,
-                                                      nullptr);
+  run_chunk<EST, XP, AP, SCHEME, PC, KP, false, false>(args, args.use_one ? &args.one : args.items, args.n_items,
+                                                      args.chunk0 + blockIdx.x, nullptr);
 }
 
 // The same for launches with per-sample records (parity runs): a kernel of
