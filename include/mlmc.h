@@ -338,7 +338,7 @@ mlmc_status mlmc_estimate(double eps, const mlmc_params *p, int mode, uint64_t s
  * completed requests.  Slots are limited by max_slots and by
  * device_bytes_budget (0 = no budget): a slot needs its state, templates and
  * work-list space, about 30 KB at max_level 10.  The per-chunk partial array
- * (48 bytes a chunk) starts at max(4 chunks per template, 65536) and grows
+ * (48 bytes a chunk) starts at max(4 chunks per template, 32768) and grows
  * when an iteration needs more.
  * Requests that share a seed must have distinct request_id values in their
  * params.  Errors: MLMC_EINVAL for bad arguments (params->formats, when

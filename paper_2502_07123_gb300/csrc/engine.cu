@@ -75,7 +75,7 @@ struct SlotReport {
 // Per (slot, level, estimator) template: what the scheduler needs beside the ItemDesc.
 struct TmplMeta {
   int32_t group;          // launch group, -1: no template
-  int32_t kp, threads, spt;
+  int32_t kp, threads, spt, grow;   // grow: chunk_count's
   int32_t unit, exact_int, level, est;
   double disc;
 };
@@ -170,7 +170,7 @@ __device__ uint64_t pending_chunks(const TmplMeta &m, unsigned long long first, 
   const uint64_t spc = samples_per_group(m.level, m.kp);
   *g0 = first / spc;
   *g1 = (first + N + spc - 1) / spc;
-  return chunk_count(*g1 - *g0, steps_per_group(m.level), m.kp, m.threads, m.spt, num_sms, gpt);
+  return chunk_count(*g1 - *g0, steps_per_group(m.level), m.kp, m.threads, m.spt, num_sms, gpt, true, m.grow != 0);
 }
 
 // One block of 1024 threads: the iteration's work list, grouped by launch group,
@@ -762,8 +762,9 @@ mlmc_status admit(mlmc_engine *e, int sl, size_t idx, cudaStream_t st) {
       int unit, ei;
       mlmc_status s = build_item(w, 0, nullptr, b, disc, unit, ei, ctx_tables());
       int th, sp, gi = -1;
+      bool grow = false;
       if (s == MLMC_OK) {
-        tuning_for(b.family, b.scheme, b.pc, l, &th, &sp);
+        grow = tuning_for(b.family, b.scheme, b.pc, l, &th, &sp);
         s = group_of(e, b, th, r.seed, &gi);
       }
       if (s != MLMC_OK) {
@@ -776,7 +777,7 @@ mlmc_status admit(mlmc_engine *e, int sl, size_t idx, cudaStream_t st) {
       const int t = l * 2 + k;
       tm[t] = b.it;
       TmplMeta &m = meta[t];
-      m.group = gi; m.kp = b.kp; m.threads = th; m.spt = sp;
+      m.group = gi; m.kp = b.kp; m.threads = th; m.spt = sp; m.grow = grow;
       m.unit = unit; m.exact_int = ei; m.level = l; m.est = k; m.disc = disc;
       gl.push_back(gi);
     }
@@ -836,7 +837,7 @@ mlmc_status mlmc_engine_create(mlmc_engine **out, const mlmc_engine_config *cfg)
   e->iters = cfg->iters_per_launch != 0 ? cfg->iters_per_launch : 1;
   e->num_sms = ctx_num_sms();
   const size_t nt = (size_t)slots * il;
-  e->cap_chunks = std::max<unsigned long long>(4ULL * nt, 1ULL << 16);
+  e->cap_chunks = std::max<unsigned long long>(4ULL * nt, 1ULL << 15);
   bool ok = dev_alloc(&e->d_slots, slots) && dev_alloc(&e->d_rep, slots) && dev_alloc(&e->d_tmpl, nt) &&
             dev_alloc(&e->d_run, nt) && dev_alloc(&e->d_meta, nt) && dev_alloc(&e->d_tnch, nt) &&
             dev_alloc(&e->d_run_nch, nt) && dev_alloc(&e->d_run_cb, nt) && dev_alloc(&e->d_run_src, nt) &&

@@ -138,7 +138,8 @@ extern std::map<std::tuple<int, int, int, int>, std::pair<int, int>> g_tune;
 extern uint64_t g_tune_gen;
 int level_class(int level);
 // Launch shape (CTA threads, fine path-steps per thread) of a kernel class.
-void tuning_for(int family, int scheme, int pc, int level, int *threads, int *spt);
+// Launch shape of a kernel class; true: the default one (chunk_count's grow).
+bool tuning_for(int family, int scheme, int pc, int level, int *threads, int *spt);
 
 // A work item with its constants and tables resolved (build_item), before
 // chunking (chunk_built).
@@ -183,7 +184,7 @@ void item_cache_clear();
 // Empty mlmc_run's cache of host-built plans (plan.cu).
 void plan_cache_clear();
 // floor: at least four CTAs per SM for this item alone (see chunk_count).
-mlmc_status chunk_built(BuiltItem &b, int threads, int spt, int num_sms, bool floor = true);
+mlmc_status chunk_built(BuiltItem &b, int threads, int spt, bool grow, int num_sms, bool floor = true);
 void make_round_keys(uint64_t seed, mlmc::RoundKeys &rk);
 // chunk kind of an item in the merged nested kernel (families 17 / 24), or -1
 int merged_kind(const BuiltItem &b);

@@ -54,10 +54,11 @@ uint64_t g_tune_gen = 0;
 
 int level_class(int level) { return level <= 1 ? level : (level <= 4 ? 2 : (level <= 7 ? 3 : 4)); }
 
-void tuning_for(int family, int scheme, int pc, int level, int *threads, int *spt) {
+bool tuning_for(int family, int scheme, int pc, int level, int *threads, int *spt) {
   auto f = g_tune.find(std::make_tuple(family, scheme, pc, level_class(level)));
   *threads = f == g_tune.end() ? TUNE_THREADS : f->second.first;
   *spt = f == g_tune.end() ? TUNE_SPT : f->second.second;
+  return f == g_tune.end();
 }
 
 // ---------------------------------------------------------------------------
@@ -406,12 +407,16 @@ int tab_y0_of(const BuiltItem &b, const void *dump) {
 }
 
 // Split an item's sample groups into chunks of `threads` x groups_per_thread.
-mlmc_status chunk_built(BuiltItem &b, int threads, int spt, int num_sms, bool floor) {
+mlmc_status chunk_built(BuiltItem &b, int threads, int spt, bool grow, int num_sms, bool floor) {
   ItemDesc &it = b.it;
   uint32_t gpt = 1;
   const uint64_t spg = steps_per_group(it.level);
-  const uint64_t nch = chunk_count(it.g1 - it.g0, spg, b.kp, threads, spt, num_sms, &gpt, floor);
-  if (nch > 0x7fffffffULL) return MLMC_EINVAL;
+  const uint64_t nch = chunk_count(it.g1 - it.g0, spg, b.kp, threads, spt, num_sms, &gpt, floor, grow);
+  // (the limit is on CTAs of the shape's own size)
+  uint32_t own = 0;
+  if (nch > 0x7fffffffULL / 2 &&
+      chunk_count(it.g1 - it.g0, spg, b.kp, threads, spt, num_sms, &own, floor, false) > 0x7fffffffULL)
+    return MLMC_EINVAL;
   it.groups_per_thread = gpt;
   it.n_chunks = (uint32_t)nch;
   b.chunk_cost = (double)gpt * (double)threads * (double)spg * b.kp * b.cost_step;

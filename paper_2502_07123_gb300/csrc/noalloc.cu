@@ -148,8 +148,11 @@ extern "C" mlmc_status mlmc_level_noalloc(int level, uint64_t N, const mlmc_para
   int unit = 0, exact_int = 0;
   if ((s = build_item(w, 0, nullptr, b, disc, unit, exact_int, src)) != MLMC_OK) return s;
   int threads, spt;
-  tuning_for(b.family, b.scheme, b.pc, level, &threads, &spt);
-  if ((s = chunk_built(b, threads, spt, nsm)) != MLMC_OK) return s;
+  const bool grow = tuning_for(b.family, b.scheme, b.pc, level, &threads, &spt);
+  // the documented limit is on CTAs of the shape's own size
+  if ((s = chunk_built(b, threads, spt, false, nsm)) != MLMC_OK) return s;
+  if (b.it.n_chunks > NOALLOC_MAX_CTAS) return MLMC_EINVAL;
+  if ((s = chunk_built(b, threads, spt, grow, nsm)) != MLMC_OK) return s;
   if (b.it.n_chunks > NOALLOC_MAX_CTAS) return MLMC_EINVAL;  // beyond the scratch array's CTA capacity
   b.it.chunk_begin = 0;
   MLMC_CK(cudaMemcpyAsync(&S->item, &b.it, sizeof(ItemDesc), cudaMemcpyHostToDevice, st));

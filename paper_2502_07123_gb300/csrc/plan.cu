@@ -232,17 +232,20 @@ mlmc_status plan_create_impl(mlmc_plan **out, const mlmc_work *work, int n_work,
     pl->N.resize(n_work);
     std::vector<BuiltItem> built(n_work);
     std::vector<int> item_threads(n_work), item_spt(n_work);
+    std::vector<char> item_grow(n_work);
     for (int i = 0; i < n_work; ++i) {
       s = build_item_cached(work[i], i, dumps ? dumps[i] : nullptr, built[i], pl->disc[i], pl->unit[i],
                             pl->exact_int[i]);
       if (s != MLMC_OK) return s;
       int th, sp;
-      tuning_for(built[i].family, built[i].scheme, built[i].pc, work[i].level, &th, &sp);
+      bool grow = tuning_for(built[i].family, built[i].scheme, built[i].pc, work[i].level, &th, &sp);
+      grow = grow && !o_threads && !o_spt;
       if (o_threads) th = o_threads;
       if (o_spt) sp = o_spt;
       item_threads[i] = th;
       item_spt[i] = sp;
-      s = chunk_built(built[i], th, sp, g.num_sms);
+      item_grow[i] = grow;
+      s = chunk_built(built[i], th, sp, grow, g.num_sms);
       if (s != MLMC_OK) return s;
       pl->N[i] = work[i].N;
       pl->path_steps += work[i].N << work[i].level;
@@ -286,7 +289,7 @@ mlmc_status plan_create_impl(mlmc_plan **out, const mlmc_work *work, int n_work,
         uint64_t total = 0;
         for (int i : kv.second) {
           alt.push_back(built[i]);
-          if ((s = chunk_built(alt.back(), item_threads[i], item_spt[i], g.num_sms, false)) != MLMC_OK) {
+          if ((s = chunk_built(alt.back(), item_threads[i], item_spt[i], item_grow[i], g.num_sms, false)) != MLMC_OK) {
             return s;
           }
           total += alt.back().it.n_chunks;
@@ -811,7 +814,7 @@ mlmc_status mlmc_autotune(const mlmc_work *work, int n_work, uint64_t seed, int 
   for (const Key &k : order) {
     const std::vector<int> &ix = cls[k];
     int cur_t, cur_s;
-    tuning_for(std::get<0>(k), std::get<1>(k), std::get<2>(k), work[ix[0]].level, &cur_t, &cur_s);
+    const bool untuned = tuning_for(std::get<0>(k), std::get<1>(k), std::get<2>(k), work[ix[0]].level, &cur_t, &cur_s);
     int best_t = cur_t, best_s = cur_s;
     double best_ms = 0.0;
     if ((s = time_plan(work, n_work, seed, reps, &best_ms)) != MLMC_OK) return s;
@@ -823,7 +826,7 @@ mlmc_status mlmc_autotune(const mlmc_work *work, int n_work, uint64_t seed, int 
           std::vector<uint32_t> sig{(uint32_t)th};
           for (int i : ix) {
             BuiltItem b = built[i];
-            if ((s = chunk_built(b, th, sp, g.num_sms)) != MLMC_OK) return s;
+            if ((s = chunk_built(b, th, sp, pass == 0 && untuned, g.num_sms)) != MLMC_OK) return s;
             sig.push_back(b.it.groups_per_thread);
           }
           if (std::find(seen.begin(), seen.end(), sig) != seen.end()) continue;
@@ -841,6 +844,7 @@ mlmc_status mlmc_autotune(const mlmc_work *work, int n_work, uint64_t seed, int 
           }
         }
     g_tune[k] = std::make_pair(best_t, best_s);
+    if (untuned && best_t == cur_t && best_s == cur_s) g_tune.erase(k);   // the default, as it was
     ++g_tune_gen;
     if (chosen)
       for (int i : ix) {
