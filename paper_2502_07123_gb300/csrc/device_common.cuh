@@ -67,38 +67,44 @@ __device__ __forceinline__ void copies_done() { asm volatile("cp.async.wait_all;
 // The inverse-Normal cubics (phi_inv_table.h) in shared memory.  A warp's 32
 // random 16-byte reads of one copy cost 10.4 wavefronts on average (the fullest
 // of 8 bank groups, per quarter warp); beside the pair table's 6.2 they held
-// shared memory 76% busy in the correction kernels.  So the parts of the six octaves [2^-7, 1/2) -- 63 of 64
-// draws -- are kept eight times, one copy per bank group, and lane l reads copy
-// l mod 8: 4 wavefronts and about half a conflict with a rarer part, which is
-// kept once.  19 KB.  8,000,009 level-4 corrections: 317 -> 297 us.
+// shared memory 76% busy in the correction kernels.  So there (OCT = 4) the parts
+// of the four octaves [2^-5, 1/2) -- 15 of 16 draws -- are kept eight times, one
+// copy per bank group, and lane l reads copy l mod 8: 4 wavefronts and about 1.7
+// conflicts with a rarer part, which is kept once.  15 KB; 8,000,009 level-4
+// corrections 317 -> 297 us.  The exact kernels, whose shared memory is 30% busy,
+// keep one copy (OCT = 0, 8 KB): staging more slowed their short chunks by 5%.
 constexpr int PHI_K0 = 94 << 4;   // exponent field and top four bits of the first part, u = 2^-33
-constexpr int PHI_HOT0 = 26 * 16, PHI_COPIES = 8;
-constexpr int PHI_SMEM = PHI_HOT0 + (PHI_INV_PARTS - PHI_HOT0) * PHI_COPIES;   // in float4
-__device__ __forceinline__ void stage_phi_inv(float4 *d) {
-  for (int k = threadIdx.x; k < PHI_HOT0; k += blockDim.x) copy16_async(d + k, k_phi_inv + k);
-  for (int k = threadIdx.x; k < PHI_SMEM - PHI_HOT0; k += blockDim.x)
-    copy16_async(d + PHI_HOT0 + k, k_phi_inv + PHI_HOT0 + k / PHI_COPIES);
-}
-// What exact_normal_f32 adds to 8 x (exponent and top bits) for the calling lane's copy.
-__device__ __forceinline__ uint32_t phi_lane() {
-  return (threadIdx.x & (PHI_COPIES - 1)) + (uint32_t)(PHI_K0 + PHI_HOT0 - PHI_COPIES * (PHI_K0 + PHI_HOT0));
-}
+template <int OCT>
+struct PhiTable {
+  static constexpr int COPIES = OCT ? 8 : 1, HOT0 = OCT ? (32 - OCT) * 16 : PHI_INV_PARTS;
+  static constexpr int SIZE = HOT0 + (PHI_INV_PARTS - HOT0) * COPIES;   // in float4
+  static __device__ __forceinline__ void stage(float4 *d) {
+    for (int k = threadIdx.x; k < HOT0; k += blockDim.x) copy16_async(d + k, k_phi_inv + k);
+    for (int k = threadIdx.x; k < SIZE - HOT0; k += blockDim.x)
+      copy16_async(d + HOT0 + k, k_phi_inv + HOT0 + k / COPIES);
+  }
+  // What a hot part's index adds to COPIES x (exponent and top bits) for the calling lane's copy.
+  static __device__ __forceinline__ uint32_t lane() {
+    return (threadIdx.x & (COPIES - 1)) + (uint32_t)(PHI_K0 + HOT0 - COPIES * (PHI_K0 + HOT0));
+  }
+};
 
 // Exact Normal Z = Phi^{-1}(2^-32 (J + 1/2)) in single precision (Sec. 3.1).
 // The upper half uses Phi^{-1}(1 - u) = -Phi^{-1}(u): with J' = J or ~J below
 // 2^31, u = 2^-32 (J' + 1/2) (J' rounded to nearest as a float) lies in
-// [2^-33, 1/2].  Phi^{-1}(u) is the cubic of u's part (tab: staged as above,
-// lane: phi_lane()): u's exponent and the top four bits of its significand
+// [2^-33, 1/2].  Phi^{-1}(u) is the cubic of u's part (tab: staged as
+// above, lane: PhiTable::lane()): u's exponent and the top four bits of its significand
 // pick one of 512 parts of [2^-33, 1/2) (the 513th is u = 1/2), the other 19
 // bits are the position t in [0, 1) within it, which as the low bits of a
 // float of [16, 17) need no shift.  Error: about 1e-7 (1 + |Z|), unbiased
 // (round to nearest).
+template <int OCT>
 __device__ __forceinline__ float exact_normal_f32(uint32_t J, const float4 *tab, uint32_t lane) {
   const uint32_t m = (uint32_t)((int32_t)J >> 31);
   const float u = fmaf(__uint2float_rn(J ^ m), 0x1p-32f, 0x1p-33f);
   const uint32_t b = __float_as_uint(u);
   uint32_t k = b >> 19;
-  if (b >= (uint32_t)(PHI_K0 + PHI_HOT0) << 19) k = k * PHI_COPIES + lane;
+  if (OCT > 0 && b >= (uint32_t)(PHI_K0 + PhiTable<OCT>::HOT0) << 19) k = k * PhiTable<OCT>::COPIES + lane;
   const float4 c = tab[(int)k - PHI_K0];
   const float t = __uint_as_float((b & 0x7FFFFu) | 0x41800000u) - 16.0f;
   const float z = fmaf(fmaf(fmaf(c.w, t, c.z), t, c.y), t, c.x);

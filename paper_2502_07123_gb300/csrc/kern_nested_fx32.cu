@@ -10,7 +10,7 @@ cudaError_t launch_nested_fx32(int scheme, int pc, dim3 grid, dim3 block, size_t
   if (scheme != 0 || pc != PC_TERMINAL || occ || a.dyn || a.dump) return cudaErrorInvalidValue;
   auto k = pre ? nested_kernel<0, PC_TERMINAL, true> : nested_kernel<0, PC_TERMINAL, false>;
   // above 48 KB of dynamic plus static shared memory (the static part holds
-  // up to about 19.6 KB: the inverse-Normal cubics) the kernel must opt in
+  // up to about 15.8 KB: the inverse-Normal cubics) the kernel must opt in
   if (smem > 24 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

@@ -74,15 +74,22 @@ template <int EST, int XP, int AP, int SCHEME, int PC, int KP, bool DYN = false>
 // The inverse-Normal cubics of the FP32 exact path in shared memory, the same
 // for every item.  Kernels whose chunks run an FP32 exact path stage them once
 // per CTA, before their first chunk's table (whose barrier makes them visible).
+template <int OCT>
 __device__ __forceinline__ float4 *phi_inv_smem() {
-  __shared__ float4 s_phi_inv[PHI_SMEM];
+  __shared__ float4 s_phi_inv[PhiTable<OCT>::SIZE];
   return s_phi_inv;
 }
+template <int OCT>
+__device__ __forceinline__ void stage_phi_inv() {
+  PhiTable<OCT>::stage(phi_inv_smem<OCT>());
+}
+constexpr int PHI_OCT_CORR = 4, PHI_OCT_EXACT = 0;
 
 // The exact path's inverse-Normal table of a kernel, if it has one.
 template <int EST, int XP>
 __device__ __forceinline__ void stage_exact_table() {
-  if constexpr (EST != EST_APPROX && XP == XP_F32) stage_phi_inv(phi_inv_smem());
+  if constexpr (EST == EST_CORR && XP == XP_F32) stage_phi_inv<PHI_OCT_CORR>();
+  if constexpr (EST == EST_EXACT && XP == XP_F32) stage_phi_inv<PHI_OCT_EXACT>();
   if constexpr (EST != EST_APPROX && XP == XP_F64) stage_phi64();
 }
 
@@ -146,6 +153,7 @@ struct LevelSim {
   static constexpr bool HAS_EXACT = (EST != EST_APPROX);
   static constexpr bool HAS_APPROX = (EST != EST_EXACT);
   static constexpr bool MIL = (SCHEME == 1);
+  static constexpr int PHI_OCT = EST == EST_CORR ? PHI_OCT_CORR : PHI_OCT_EXACT;
   static constexpr bool PERM = EST == EST_CORR && MSEL >= 2;   // Method 2's coupling of the exact path
   static constexpr bool FAST = (AP == AP_FX32 || AP == AP_FX64);
   static constexpr bool FIXED = (AP == AP_FIXED || FAST);
@@ -190,7 +198,7 @@ struct LevelSim {
   uint32_t rot[KP], off_mask;
   const uint16_t *perm_s;  // method 2 coupling of the exact path (shared memory), or nullptr
   const float4 *phi;       // FP32 exact path: the inverse-Normal cubics in shared memory
-  uint32_t phil;           // and this lane's copy (phi_lane)
+  uint32_t phil;           // and this lane's copy (PhiTable::lane)
   uint32_t low_mask;
   X c1, c2, c1c, c3, S0, K;
   // FP64 exact path: integer increments (exact64.cuh)
@@ -268,8 +276,8 @@ struct LevelSim {
     }
     perm_s = nullptr;
     if constexpr (HAS_EXACT && XP == XP_F32) {
-      phi = phi_inv_smem();
-      phil = phi_lane();
+      phi = phi_inv_smem<PHI_OCT>();
+      phil = PhiTable<PHI_OCT>::lane();
     }
     low_mask = (1u << dshift) - 1u;
     if constexpr (PERM) {
@@ -521,7 +529,7 @@ struct LevelSim {
           inc = exact_inc(z, c1, X(1));
         }
       } else {
-        z = exact_normal_f32(Je, phi, phil);
+        z = exact_normal_f32<PHI_OCT>(Je, phi, phil);
         inc = exact_inc(z, c1, X(1));
       }
       if constexpr (PC == PC_ASIAN) { if (i > 0) accF = accF + S; }
@@ -1381,7 +1389,9 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
     const int n = 1 << d;
     // merged launch: only the correction chunks (kind 2) run the FP32 exact path;
     // the copies proceed while the pairs are formed
-    if (PHI_BY_KIND && it.kind == 2) stage_phi_inv(phi_inv_smem());
+    if constexpr (PHI_BY_KIND) {
+      if (it.kind == 2) stage_phi_inv<PHI_OCT_CORR>();
+    }
     const bool pre = fx32_pre(it), p32 = pre && SCHEME == 0;
     int2 *dst = (int2 *)smem_tab;
     int32_t *dst4 = (int32_t *)smem_tab;
@@ -1565,7 +1575,7 @@ cudaError_t launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t st, cons
             : a.dump       ? level_kernel_dump<EST, XP, AP, SCHEME, PC, KP>
                            : level_kernel<EST, XP, AP, SCHEME, PC, KP>;
   // above 48 KB of dynamic plus static shared memory (the static part holds
-  // up to about 19.6 KB: the inverse-Normal cubics) the kernel must opt in
+  // up to about 16.6 KB: the inverse-Normal cubics) the kernel must opt in
   if (smem > 24 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;

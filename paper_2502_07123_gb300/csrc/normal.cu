@@ -13,14 +13,13 @@ using namespace mlmc;
 namespace {
 
 __global__ void exact_normal_kernel(const uint32_t *J, float *z, uint64_t n) {
-  __shared__ float4 tab[PHI_SMEM];
-  stage_phi_inv(tab);
+  __shared__ float4 tab[PhiTable<0>::SIZE];
+  PhiTable<0>::stage(tab);
   copies_done();
   __syncthreads();
-  const uint32_t lane = phi_lane();
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-    z[i] = exact_normal_f32(J[i], tab, lane);
+    z[i] = exact_normal_f32<0>(J[i], tab, 0);
 }
 
 }  // namespace
