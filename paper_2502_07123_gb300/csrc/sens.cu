@@ -22,9 +22,9 @@
 // global memory (32 bytes at a time; it stays in L2 up to level 6 or so).  Pass
 // 2, a thread per instance, adds the squares over the CTA's samples: no
 // cross-lane sums, and the tape read in rows.  The per-type moments are sums of
-// the per-instance ones.  About 40 FP64 operations per path-step against 258
+// the per-instance ones.  About 25 FP64 operations per path-step against 258
 // (two library Phi^-1, four divisions, 64-bit butterflies): 100,001 level-6
-// samples 3.31 -> 0.49 ms, the FP64 unit 85% busy in both.
+// samples 3.89 -> 0.42 ms a call, the FP64 unit 85 and 74% busy.
 // Per-CTA partials are summed in CTA order by sens_finalize_kernel.
 #include <cuda_runtime.h>
 
@@ -124,6 +124,7 @@ __global__ void __launch_bounds__(SENS_THREADS, 4) sens_kernel(const SensConsts 
   long long z_hi = -0x7FFFFFFFFFFFFFFFLL, z_lo = 0x7FFFFFFFFFFFFFFFLL, zc_hi = z_hi, zc_lo = z_lo;
   const uint64_t stride = (uint64_t)gridDim.x * SENS_THREADS;
   for (int it = 0; it < iters; ++it) {
+    if ((uint64_t)it * stride + (uint64_t)blockIdx.x * SENS_THREADS >= c.N) break;   // no sample for this CTA
     const uint64_t rel = (uint64_t)it * stride + (uint64_t)blockIdx.x * SENS_THREADS + tid;
     const bool valid = rel < c.N;
     const uint64_t s = c.first + (valid ? rel : 0);
@@ -351,9 +352,11 @@ extern "C" mlmc_status mlmc_sensitivities(int level, uint64_t N, const mlmc_para
     exact64_consts(it, false);
     c.q1 = it.q1; c.q2 = it.q2; c.qF = it.qF;
   }
-  // four CTAs per SM where the tape allows
+  // a CTA per 128 samples while their tapes fit the kept workspace, at least the
+  // four per SM that run at once (where the tape allows)
   const size_t tape = sizeof(double) * tape_doubles(c.n, c.m);
-  const uint64_t want = std::min<uint64_t>((uint64_t)4 * ctx_num_sms(), SENS_MAX_TAPE / tape);
+  const uint64_t want = std::max<uint64_t>(std::min<uint64_t>((uint64_t)4 * ctx_num_sms(), SENS_MAX_TAPE / tape),
+                                           (SENS_KEEP - SENS_KEEP / 8) / tape);
   const int n_ctas = (int)std::min<uint64_t>(want, (N + SENS_THREADS - 1) / SENS_THREADS);
   const uint64_t per = (uint64_t)n_ctas * SENS_THREADS;
   const int iters = (int)((N + per - 1) / per);
