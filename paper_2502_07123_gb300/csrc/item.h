@@ -88,6 +88,7 @@ struct ItemDesc {
   int32_t tab_y0;          // 1: a level-0 approximate item of the 32-bit fast datapath with a terminal
                            // payoff; its shared-memory table holds Y_j, the sample value of every
                            // index j (its one fine step is a function of j alone)
+  int32_t y0_bits;         // there: 2^y0_bits samples' Y^2 fit in 64 bits
   float unit_scale;        // 2^-unit (FP32, correction estimators)
   // exact path constants
   float c1f, c2f, c1cf, c3f, S0f, Kf;

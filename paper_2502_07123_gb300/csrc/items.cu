@@ -401,6 +401,11 @@ int64_t table_zmax_fixed(const double *Z, int d, int method, int fZ, int fields)
 // (tab_y0), unless they write per-sample records.  Only lazy items: S_0 <=
 // limT there, so no index's one fine step leaves lim_S and no sample counts a
 // saturation (the items that may saturate keep the clamped step code).
+int bit_length(uint64_t x) {
+  int n = 0;
+  for (; x; x >>= 1) ++n;
+  return n;
+}
 int tab_y0_of(const BuiltItem &b, const void *dump) {
   return (b.family == 8 || b.family == 15) && b.it.level == 0 && b.pc == PC_TERMINAL && b.it.ff.lazy && !dump ? 1
                                                                                                               : 0;
@@ -640,6 +645,9 @@ mlmc_status build_item(const mlmc_work &w, int out_index, void *dump, BuiltItem 
   b.scheme = p->scheme;
   b.pc = p->payoff == MLMC_ASIAN ? PC_ASIAN : (p->payoff == MLMC_LOOKBACK ? PC_LOOKBACK : PC_TERMINAL);
   it.tab_y0 = tab_y0_of(b, dump);
+  // |Y| <= max(lim_S, 2^f_S) < 2^ybits
+  const int ybits = std::max(bit_length((uint64_t)it.ff.limS), it.fx.fS + 1);
+  it.y0_bits = std::max(0, 64 - 2 * ybits);
   return MLMC_OK;
 }
 

@@ -373,30 +373,27 @@ struct LevelSim {
   __device__ __forceinline__ AS ff_step(AS s, int32_t z, int32_t c1r, int64_t m, SatT &satb) {
     return ff_apply<EAGER>(s, ff_sum1<MIL, AP == AP_FX32>(ff, z, c1r, m), satb);
   }
-  // FX32: byte offset of lane l's table entry for word w.  Lane 0's field (and
-  // the only one of an unpacked word) is the top one: no mask.
-  __device__ __forceinline__ uint32_t fx32_off(uint32_t w, int l) const {
-    if (l == 0) return (w >> dshift) << LG;
-    return __funnelshift_r(w, w, rot[l]) & off_mask;
-  }
-  // The table sits at the start of the dynamic shared memory: addressing it
-  // there, rather than through smem_tab, leaves the base to the load's
-  // immediate offset, one add fewer per lookup.
-  template <class E>
-  __device__ __forceinline__ E fx32_entry(uint32_t off) const {
+  // FX32: lane l's table entry for word w.  Lane 0's field (and the only one of an
+  // unpacked word) is the top one: no mask.  The table sits at the start of the
+  // dynamic shared memory: addressing it there, rather than through smem_tab,
+  // leaves the base to the load's immediate offset, one add fewer per lookup.
+  // SH: log2 of the entry's bytes in the table read.
+  template <class E, int SH = LG>
+  __device__ __forceinline__ E fx32_entry(uint32_t w, int l) const {
     extern __shared__ __align__(16) unsigned char smem_dyn[];
-    return *(const E *)(smem_dyn + off);
+    if (l == 0) return ((const E *)smem_dyn)[w >> dshift];
+    return *(const E *)(smem_dyn + ((__funnelshift_r(w, w, rot[l]) & off_mask) >> (LG - SH)));
   }
   // The FX32 fine step of lane l on word w; returns what the coarse step needs of
   // it (Z~, or P_j).  TRACK as in ff_apply.
   template <bool EAGER, bool TRACK>
   __device__ __forceinline__ int32_t fx32_fine(uint32_t w, int l) {
     if constexpr (P32) {
-      const int32_t q = fx32_entry<int32_t>(fx32_off(w, l));
+      const int32_t q = fx32_entry<int32_t>(w, l);
       aS[l] = ff_apply<EAGER, TRACK>(aS[l], (q >> ff.rs1) * pre2 + c1p, satb[l]);
       return q;
     } else {
-      const int2 e = fx32_entry<int2>(fx32_off(w, l));
+      const int2 e = fx32_entry<int2>(w, l);
       aS[l] = ff_apply<EAGER, TRACK>(aS[l], e.y, satb[l]);
       return e.x;
     }
@@ -1106,26 +1103,31 @@ __device__ __forceinline__ void y0_group(const Sim &sim, Acc &acc, const uint4 &
 #pragma unroll
     for (int l = 0; l < KP; ++l) {
       const int k = u * KP + l;
-      y[k] = sim.template fx32_entry<int32_t>(sim.fx32_off(word_of(w, u), l) >> (Sim::LG - 2));
+      y[k] = sim.template fx32_entry<int32_t, 2>(word_of(w, u), l);
       if (!(FULL || (k >= klo && k < khi))) y[k] = 0;
     }
   }
 #pragma unroll
   for (int k = 0; k < 4 * KP; k += 2) acc.add_group2(y[k], y[k + 1]);
-  acc.flush_group();
 }
 
 // The groups of a chunk of such an item: the same samples and values as
 // run_group's path (no saturation: see tab_y0_of).
 template <class Sim, class Acc>
 __device__ __forceinline__ void group_loop_y0(const Sim &sim, Acc &acc, const LaunchArgs &args, const GroupCtx &it,
-                                              uint64_t gbeg, uint32_t ng, uint32_t rf0, uint32_t rf1) {
+                                              uint64_t gbeg, uint32_t ng, uint32_t rf0, uint32_t rf1, bool once) {
   constexpr int KP = Sim::KPV;
   const uint64_t first = it.first, last = it.last;
+  // the chunk's Philox calls share the counter's high word but for one in 2^32;
+  // once: a thread's whole sums stay in the 64-bit group sums, where they fit
+  const uint32_t hi = (uint32_t)(gbeg >> 32);
+  const bool one_hi = (uint32_t)((gbeg + ng) >> 32) == hi;
+  const PhiloxStream ps(hi, it.ctr2, it.ctr3, args.rk);
   for (uint32_t r = threadIdx.x; r < ng; r += blockDim.x) {
     const uint64_t g = gbeg + r;
     uint4 w;
     if (Sim::ENUMERATE && it.enumerate) w = enum_words(g, 0, it.d);
+    else if (one_hi) w = ps.call((uint32_t)g, args.rk);
     else w = draw(it, args, g);
     if (r >= rf0 && r < rf1) {
       y0_group<true>(sim, acc, w, 0, 0);
@@ -1135,7 +1137,9 @@ __device__ __forceinline__ void group_loop_y0(const Sim &sim, Acc &acc, const La
       const int khi = last <= s0 ? 0 : (int)min(last - s0, (uint64_t)(4 * KP));
       y0_group<false>(sim, acc, w, klo, khi);
     }
+    if (!once) acc.flush_group();
   }
+  acc.flush_group();
 }
 
 // A thread's groups of one chunk, groups gbeg + r for r = threadIdx.x,
@@ -1286,7 +1290,11 @@ __device__ __forceinline__ void chunk_body(const LaunchArgs &args, const ItemDes
     const bool y0 = EST == EST_APPROX && it.tab_y0;
     if (lc == 0) {
       if (y0) {
-        if constexpr (EST == EST_APPROX) group_loop_y0(sim, acc, args, gx, gbeg, ng, rf0, rf1);
+        if constexpr (EST == EST_APPROX) {
+          // samples of a thread (at most) times y^2 < 2^64
+          const uint64_t most = (uint64_t)it.groups_per_thread * (4u * KP);
+          group_loop_y0(sim, acc, args, gx, gbeg, ng, rf0, rf1, it.y0_bits < 64 && most <= (1ULL << it.y0_bits));
+        }
       }
       else if (dig) loop(L0{}, PayTag<1>{});
       else loop(L0{}, PayTag<0>{});
