@@ -756,7 +756,8 @@ struct LevelSim {
   // Finish the sample: payoffs, sample value, accumulation and optional dump
   // (EAGER false: a LAZY pack that stayed in range, so no saturation).
   // LV: 0 on level 0 (no coarse path), 1 on levels >= 1, -1 not known at compile time.
-  template <bool EAGER = true, int PAY = -1, int LV = -1, class Acc>
+  // PAIRED: real samples are taken two at a time (levels 0 and 1; ThreadAcc).
+  template <bool EAGER = true, int PAY = -1, int LV = -1, bool PAIRED = false, class Acc>
   __device__ __forceinline__ void finish(Acc &acc, int l, bool valid, mlmc_sample_rec *dump) {
     X pf = X(0), pc = X(0);
     int64_t qf = 0, qc = 0, afS = 0, acS = 0;
@@ -800,13 +801,13 @@ struct LevelSim {
       // a sample outside the item's range adds zero: no branch
       if constexpr (EST == EST_EXACT) {
         const X y = valid ? pf - pc : X(0);
-        acc.add_real(y);
+        acc.template add_real<PAIRED>(y);
         ydump = (double)y;
       } else {
         const float yx = (float)(pf - pc);
         const float ya = __fmul_rn(__ll2float_rn(qf - qc), unit_scale);
         const float y = valid ? __fsub_rn(yx, ya) : 0.0f;
-        acc.add_real(y);
+        acc.template add_real<PAIRED>(y);
         ydump = (double)y;
       }
       acc.nsat += valid ? lsat : 0u;
@@ -832,9 +833,39 @@ struct LevelSim {
   }
 };
 
+// Two floats in one 64-bit register pair and the instructions on both at once
+// (each result rounded as the scalar operation's): half the issue slots.
+struct F2 {
+  uint64_t v;
+  static __device__ __forceinline__ F2 of(float a, float b) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(a), "f"(b));
+    return r;
+  }
+  __device__ __forceinline__ void get(float &a, float &b) const { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+};
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+// a - b, exactly as a subtraction: -1 b + a is one rounding of a - b.
+__device__ __forceinline__ F2 sub2(F2 a, F2 b) { return fma2(F2{0xBF800000BF800000ULL}, b, a); }
+
 // Samples of an FP32 real-valued estimator summed in a float pair before each
-// FP64 flush (see ThreadAcc::add_real).
-constexpr int REAL_FLUSH_SAMPLES = 8;
+// FP64 flush: levels >= 2, and pairs of samples on levels 0 and 1 (see
+// ThreadAcc::add_real).
+constexpr int REAL_FLUSH_SAMPLES = 8, REAL_FLUSH_PAIRS = 6;
 
 // Per-thread accumulator
 template <int EST, int XP>
@@ -845,12 +876,17 @@ struct ThreadAcc {
   // real-valued estimators: FP64 sums (FP64 exact path: every sample; FP32
   // paths and corrections: the float pairs below, flushed)
   double ds, dq;
-  // float pairs (s + c) of sum Y and sum Y^2 since the last flush
-  float fs, fc, fs2, fc2;
+  // float pairs (s + c) of sum Y and sum Y^2 since the last flush: one of each
+  // (os, oc, os2, oc2), or two, of every first and of every second sample
+  float os, oc, os2, oc2;
+  F2 fs, fc, fs2, fc2;
+  float first;             // a first sample that waits for its second (have)
+  bool have;
   uint32_t nsat;
   __device__ __forceinline__ void init() {
     isum = 0; q_lo = 0; q_hi = 0; gsum = 0; gq = 0; ds = 0.0; dq = 0.0; nsat = 0;
-    fs = 0.0f; fc = 0.0f; fs2 = 0.0f; fc2 = 0.0f;
+    os = 0.0f; oc = 0.0f; os2 = 0.0f; oc2 = 0.0f;
+    fs = F2{0}; fc = fs; fs2 = fs; fc2 = fs; first = 0.0f; have = false;
   }
   __device__ __forceinline__ void add_int(int64_t y) {
     isum += y;
@@ -886,14 +922,22 @@ struct ThreadAcc {
   struct Mark {
     int64_t isum;
     uint64_t q_lo, q_hi;
-    float fs, fc, fs2, fc2;
+    F2 fs, fc, fs2, fc2;
   };
+  // (a group of levels 0 and 1 has an even number of samples: none waits there)
   __device__ __forceinline__ Mark mark() const { return Mark{isum, q_lo, q_hi, fs, fc, fs2, fc2}; }
   __device__ __forceinline__ void rewind(const Mark &m) {
     isum = m.isum; q_lo = m.q_lo; q_hi = m.q_hi;
-    fs = m.fs; fc = m.fc; fs2 = m.fs2; fc2 = m.fc2;
+    fs = m.fs; fc = m.fc; fs2 = m.fs2; fc2 = m.fc2; have = false;
   }
   // s + y = t + e exactly (Knuth's TwoSum, six FP32 operations): s becomes t, e is returned.
+  static __device__ __forceinline__ F2 two_sum(F2 &s, F2 y) {
+    const F2 t = add2(s, y);
+    const F2 z = sub2(t, s);
+    const F2 e = add2(sub2(s, sub2(t, z)), sub2(y, z));
+    s = t;
+    return e;
+  }
   static __device__ __forceinline__ float two_sum(float &s, float y) {
     const float t = __fadd_rn(s, y);
     const float z = __fsub_rn(t, s);
@@ -901,37 +945,76 @@ struct ThreadAcc {
     s = t;
     return e;
   }
-  // A real sample.  FP64 samples are added in FP64.  An FP32 sample y enters
-  // the float pair (fs, fc) by TwoSum, so fs + fc misses sum y only by the
-  // roundings of the additions into fc; y^2 = p + pe exactly (p = fl(y y),
-  // pe = fma(y, y, -p)) enters (fs2, fc2) the same way.  With at most K =
-  // REAL_FLUSH_SAMPLES samples between flushes (|fc| <= k u sum |y| after k of
-  // them, |fc2| <= (k+1) u sum y^2, u = 2^-24) those roundings total at most
-  // u^2 K(K+1)/2 sum |y| and 2 u^2 (K(K+1)/2 + K) sum y^2: below 1.3e-13 of
-  // sum |y| and 3.2e-13 of sum y^2.  A flush adds each float, exactly widened,
-  // into the FP64 sums, so the thread's sums are within about 3.5e-13 of the
-  // exact sums of its samples, at one FP64 operation per sample.
-  template <class T>
+  // A real sample.  FP64 samples are added in FP64.  An FP32 sample y enters the
+  // float pair (os, oc) by TwoSum, so os + oc misses sum y only by the roundings
+  // of the additions into oc; y^2 = p + pe exactly (p = fl(y y), pe = fma(y, y,
+  // -p)) enters (os2, oc2) the same way.  With at most K = REAL_FLUSH_SAMPLES
+  // samples between flushes (|oc| <= k u sum |y| after k of them, |oc2| <= (k+1) u
+  // sum y^2, u = 2^-24) those roundings total at most u^2 K(K+1)/2 sum |y| and
+  // 2 u^2 (K(K+1)/2 + K) sum y^2: below 1.3e-13 of sum |y| and 3.2e-13 of sum
+  // y^2.  A flush adds each float, exactly widened, into the FP64 sums, so the
+  // thread's sums are within about 3.5e-13 of the exact sums of its samples, at
+  // one FP64 operation per sample.
+  //
+  // PAIRED (levels 0 and 1, where that is what bounds the kernel): two samples at
+  // a time, each in its own pair of (fs, fc), on two-float instructions.  After K
+  // = REAL_FLUSH_PAIRS a flush joins the two pairs of each sum by one more TwoSum,
+  // whose error and the two companions are added (2 roundings of at most (2K+1) u
+  // sum |y|), and adds two floats to the FP64 sum: at most u^2 (K(K+1)/2 + 2K + 1)
+  // sum |y| and 2 u^2 (K(K+1)/2 + K + 2K + 3) sum y^2, below 1.3e-13 and 3.1e-13.
+  // 9 instructions and 2/3 of an FP64 operation per sample, against 17 and one:
+  // 67,108,864 level-0 FP32 samples 172 -> 159 us, the FP64 unit 73 -> 54% busy.
+  template <bool PAIRED, class T>
   __device__ __forceinline__ void add_real(T y) {
     if constexpr (XP == XP_F64 && EST == EST_EXACT) {
       ds += (double)y;
       dq = fma((double)y, (double)y, dq);
+    } else if constexpr (PAIRED) {
+      if (have) add_pair(F2::of(first, (float)y));
+      first = (float)y;
+      have = !have;
     } else {
       const float yf = (float)y;
-      fc = __fadd_rn(fc, two_sum(fs, yf));
+      oc = __fadd_rn(oc, two_sum(os, yf));
       const float p = __fmul_rn(yf, yf);
       const float pe = __fmaf_rn(yf, yf, -p);
-      fc2 = __fadd_rn(__fadd_rn(fc2, two_sum(fs2, p)), pe);
+      oc2 = __fadd_rn(__fadd_rn(oc2, two_sum(os2, p)), pe);
     }
   }
+  __device__ __forceinline__ void add_pair(F2 y) {
+    fc = add2(fc, two_sum(fs, y));
+    const F2 p = mul2(y, y);
+    const F2 pe = fma2(y, y, sub2(F2{0}, p));
+    fc2 = add2(add2(fc2, two_sum(fs2, p)), pe);
+  }
   static constexpr bool PAIRS = EST != EST_APPROX && !(XP == XP_F64 && EST == EST_EXACT);
+  static __device__ __forceinline__ void flush_pair(F2 &s, F2 &c, double &d) {
+    float a, b, ca, cb;
+    s.get(a, b);
+    c.get(ca, cb);
+    const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+    if (fabsf(t) <= 3.402823466e38f) {
+      d += (double)t;
+      d += (double)__fadd_rn(__fadd_rn(ca, cb), e);
+    } else {   // the two sums together leave the float range
+      d += (double)a + (double)ca;
+      d += (double)b + (double)cb;
+    }
+    s = F2{0};
+    c = F2{0};
+  }
+  template <bool PAIRED>
   __device__ __forceinline__ void flush_real() {
-    if constexpr (PAIRS) {
-      ds += (double)fs;
-      ds += (double)fc;
-      dq += (double)fs2;
-      dq += (double)fc2;
-      fs = 0.0f; fc = 0.0f; fs2 = 0.0f; fc2 = 0.0f;
+    if constexpr (PAIRS && PAIRED) {
+      flush_pair(fs, fc, ds);
+      flush_pair(fs2, fc2, dq);
+    } else if constexpr (PAIRS) {
+      ds += (double)os;
+      ds += (double)oc;
+      dq += (double)os2;
+      dq += (double)oc2;
+      os = 0.0f; oc = 0.0f; os2 = 0.0f; oc2 = 0.0f;
     }
   }
 };
@@ -1072,7 +1155,7 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
         for (int l = 0; l < KP; ++l) {
           const int k = u * KP + l;
           const bool valid = FULL || (k >= klo && k < khi);
-          sim.template finish<E, PAY, 1>(acc, l, valid, DUMP && valid ? dump + (s0 + k - first) : nullptr);
+          sim.template finish<E, PAY, 1, true>(acc, l, valid, DUMP && valid ? dump + (s0 + k - first) : nullptr);
         }
       }
     } else {
@@ -1084,7 +1167,7 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
         for (int l = 0; l < KP; ++l) {
           const int k = u * KP + l;
           const bool valid = FULL || (k >= klo && k < khi);
-          sim.template finish<E, PAY, 0>(acc, l, valid, DUMP && valid ? dump + (s0 + k - first) : nullptr);
+          sim.template finish<E, PAY, 0, true>(acc, l, valid, DUMP && valid ? dump + (s0 + k - first) : nullptr);
         }
       }
     }
@@ -1153,11 +1236,11 @@ __device__ __forceinline__ void group_loop(Sim &sim, ThreadAcc<EST, XP> &acc, co
                                            const GroupCtx &it, uint64_t gbeg, uint32_t ng, uint32_t rf0, uint32_t rf1,
                                            bool lazy, mlmc_sample_rec *dump) {
   const uint64_t first = it.first, last = it.last;
-  // Real-valued estimators flush their float pairs every `flush_groups`
-  // groups (at most REAL_FLUSH_SAMPLES samples).
-  constexpr bool REAL = EST != EST_APPROX && !(XP == XP_F64 && EST == EST_EXACT);
+  // Real-valued estimators flush their float pairs every FLUSH_GROUPS groups
+  // (8 samples, or 6 pairs; a group of levels 0 and 1 has an even number of samples).
+  constexpr bool REAL = ThreadAcc<EST, XP>::PAIRS;
   constexpr uint32_t FLUSH_GROUPS =
-      REAL ? (uint32_t)REAL_FLUSH_SAMPLES / (uint32_t)(Sim::KPV * (LC == 2 ? 1 : (LC == 1 ? 2 : 4))) : 0u;
+      LC == 2 ? (uint32_t)REAL_FLUSH_SAMPLES : (uint32_t)REAL_FLUSH_PAIRS / (LC == 1 ? 1u : 2u);
   uint32_t since_flush = 0;
   for (uint32_t r = threadIdx.x; r < ng; r += blockDim.x) {
     const uint64_t g = gbeg + r;
@@ -1197,12 +1280,12 @@ __device__ __forceinline__ void group_loop(Sim &sim, ThreadAcc<EST, XP> &acc, co
     if constexpr (EST == EST_APPROX && AP == AP_FX32 && PC == PC_TERMINAL) acc.flush_group();
     if constexpr (REAL) {
       if (++since_flush == FLUSH_GROUPS) {
-        acc.flush_real();
+        acc.template flush_real<LC != 2>();
         since_flush = 0;
       }
     }
   }
-  acc.flush_real();
+  acc.template flush_real<LC != 2>();
 }
 
 // The first ng groups of a chunk, a multiple of 2 blockDim.x, two at a time
