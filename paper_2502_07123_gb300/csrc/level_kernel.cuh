@@ -44,12 +44,12 @@ template <> struct HType<AP_BF16S> { using T = __nv_bfloat16; };
 
 constexpr int MAX_THREADS = 256;
 // Register budget: the approximate fixed-point Euler kernel with terminal payoffs
-// (the bulk of the nested estimator) runs with 6 resident 128-thread CTAs per SM
-// (80 registers per thread), measured faster than its natural ~100 registers.
-// The matching correction kernel (static launch) takes the same budget, 80
-// instead of 111 registers: alone it is 2% slower, but beside the approximate
-// kernels of a work list its CTAs fit next to theirs and the step is 3% faster
-// (its device-scheduled form would spill there and keeps its allocation).
+// (the bulk of the nested estimator) and the merged nested kernel run with 7
+// resident 128-thread CTAs per SM (72 registers per thread, no spills): 2e8
+// packed path-steps at level 4 172 us with 6, 158 with 7 and with 8 (64
+// registers, which spill and cost level 2 1%).  The matching correction kernel
+// (static launch) takes 6, 80 registers instead of 111 (its device-scheduled
+// form would spill there and keeps its allocation); 5 cost it 0.5%.
 // The approximate 32-bit fixed-point Asian kernels run 4 CTAs per SM (<= 128
 // registers, measured 8-16% faster than their natural ~144), as do the
 // corrections whose natural allocation lies just above.
@@ -63,7 +63,8 @@ template <int EST, int XP, int AP, int SCHEME, int PC, int KP, bool DYN = false>
   static constexpr bool EM_TERMINAL_FX32 = AP == AP_FX32 && SCHEME == 0 && PC == PC_TERMINAL;
   static constexpr bool FX = AP == AP_FX32 || AP == AP_FX64;
   static constexpr int value =
-      EM_TERMINAL_FX32 && (EST == EST_APPROX || (EST == EST_CORR && !DYN)) ? 6
+      EM_TERMINAL_FX32 && EST == EST_APPROX ? 7
+      : EM_TERMINAL_FX32 && EST == EST_CORR && !DYN ? 6
       : EST == EST_EXACT && XP == XP_F32 ? (!DYN || (SCHEME == 0 && PC != PC_ASIAN) ? 6 : 1)
       : EST == EST_CORR && FX ? 4
       : EST == EST_CORR && AP != AP_FIXED && !DYN ? (SCHEME == 1 && PC == PC_ASIAN ? 4 : 5)
@@ -154,6 +155,9 @@ struct LevelSim {
   static constexpr bool HAS_APPROX = (EST != EST_EXACT);
   static constexpr bool MIL = (SCHEME == 1);
   static constexpr int PHI_OCT = EST == EST_CORR ? PHI_OCT_CORR : PHI_OCT_EXACT;
+  // the calls of a path share the first Philox rounds' constants (PhiloxStream);
+  // most packed kernels, whose calls feed three samples, keep the registers
+  static constexpr bool STREAM = KP == 1 || (AP == AP_FX32 && SCHEME == 0 && PC == PC_TERMINAL);
   static constexpr bool PERM = EST == EST_CORR && MSEL >= 2;   // Method 2's coupling of the exact path
   static constexpr bool FAST = (AP == AP_FX32 || AP == AP_FX64);
   static constexpr bool FIXED = (AP == AP_FIXED || FAST);
@@ -1112,11 +1116,10 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
     uint64_t qbase = P * calls;
     if constexpr (E && Sim::LAZY) opaque(qbase);
     sim.begin();
-    // qbase is a multiple of calls (a power of two): the calls share its high
-    // word (packed draws, whose calls feed three samples, keep the registers)
+    // qbase is a multiple of calls (a power of two): the calls share its high word
     const PhiloxStream ps((uint32_t)(qbase >> 32), it.ctr2, it.ctr3, args.rk);
     for (uint32_t c = 0; c < calls; ++c) {
-      const uint4 w = KP == 1 ? ps.call((uint32_t)qbase + c, args.rk) : draw(it, args, qbase + c);
+      const uint4 w = Sim::STREAM ? ps.call((uint32_t)qbase + c, args.rk) : draw(it, args, qbase + c);
       const int i0 = (int)(c << 2);
       sim.template step<true, 0, E>(w.x << lsh, i0);
       sim.template step<true, 1, E>(w.y << lsh, i0 + 1);
@@ -1637,7 +1640,7 @@ level_kernel_dyn(const __grid_constant__ LaunchArgs args) {
 // short chunks of every family fill in behind them.
 // PRE: every item takes the pre-scaled form (family 24; else family 17).
 template <int SCHEME, int PC, bool PRE>
-__global__ void __launch_bounds__(LAUNCH_THREADS, 6) nested_kernel(const __grid_constant__ LaunchArgs args) {
+__global__ void __launch_bounds__(LAUNCH_THREADS, 7) nested_kernel(const __grid_constant__ LaunchArgs args) {
   extern __shared__ __align__(16) unsigned char smem_tab[];
   const uint32_t gc = args.chunk0 + blockIdx.x;
   const int item = stage_chunk<AP_FX32, SCHEME, true>(args.items, args.n_items, gc, nullptr);
