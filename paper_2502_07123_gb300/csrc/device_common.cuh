@@ -111,13 +111,6 @@ __device__ __forceinline__ float exact_normal_f32(uint32_t J, const float4 *tab,
   return __uint_as_float(__float_as_uint(z) ^ (J & 0x80000000u));
 }
 
-__device__ __forceinline__ double exact_normal_f64(uint32_t J) {
-  const uint32_t m = (uint32_t)((int32_t)J >> 31);
-  const double u = ((double)(J ^ m) + 0.5) * 0x1p-32;
-  const double z = normcdfinv(u);
-  return m ? -z : z;
-}
-
 // Table index of the approximate Normal (Sec. 3.1): j = top d bits of J; the
 // upper half (leading bit of j set) mirrors the index and flips the sign, so
 // Z~ is the mean of Phi^{-1} over the 2^-d interval containing U.
