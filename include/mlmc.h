@@ -430,7 +430,10 @@ mlmc_status mlmc_batch_estimate(const mlmc_params *params, const double *eps, in
  * per instance: mul1 / sum1 / mul2: fine step k at k, coarse step k at
  * 2^l + k; S: S_{k+1} fine at k, coarse at 2^l + k, S0 last; Z: Z_j at j;
  * con1: fine 0, coarse 1; con2: 0.  level 0..10, European payoff and Euler
- * scheme only (MLMC_EINVAL otherwise).  Synchronous; allocates scratch. */
+ * scheme only (MLMC_EINVAL otherwise).  Synchronous.  Device scratch: 2 KB per
+ * fine and coarse step and CTA of 128 samples, 1.07 GB at most (level 10, from
+ * 43,521 samples); where the device has less room, fewer CTAs, down to one's 3 MB
+ * (MLMC_ENOMEM below that).  Up to 128 MB of it stay allocated for the next call. */
 typedef struct {
   double A[7];
   double B[7];

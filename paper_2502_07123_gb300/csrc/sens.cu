@@ -102,7 +102,7 @@ __host__ __device__ inline size_t tape_doubles(int n, int m) { return (size_t)SE
 // each with the samples of its residue).
 __host__ __device__ inline int slots(int n) { return n > SENS_THREADS ? n : SENS_THREADS; }
 
-__global__ void __launch_bounds__(SENS_THREADS, 4) sens_kernel(const SensConsts c, const RoundKeys rk, int iters,
+__global__ void __launch_bounds__(SENS_THREADS, 4) sens_kernel(const SensConsts c, const RoundKeys rk, uint64_t iters,
                                                             double *part, double *inst_part, double *tapes) {
   extern __shared__ double acc[];
   __shared__ double sF[SENS_THREADS], sG[SENS_THREADS], wp[P_COUNT][SENS_THREADS / 32];
@@ -123,9 +123,9 @@ __global__ void __launch_bounds__(SENS_THREADS, 4) sens_kernel(const SensConsts 
   // sample of its own repeats sample `first`, which changes no extreme
   long long z_hi = -0x7FFFFFFFFFFFFFFFLL, z_lo = 0x7FFFFFFFFFFFFFFFLL, zc_hi = z_hi, zc_lo = z_lo;
   const uint64_t stride = (uint64_t)gridDim.x * SENS_THREADS;
-  for (int it = 0; it < iters; ++it) {
-    if ((uint64_t)it * stride + (uint64_t)blockIdx.x * SENS_THREADS >= c.N) break;   // no sample for this CTA
-    const uint64_t rel = (uint64_t)it * stride + (uint64_t)blockIdx.x * SENS_THREADS + tid;
+  for (uint64_t it = 0; it < iters; ++it) {
+    if (it * stride + (uint64_t)blockIdx.x * SENS_THREADS >= c.N) break;   // no sample for this CTA
+    const uint64_t rel = it * stride + (uint64_t)blockIdx.x * SENS_THREADS + tid;
     const bool valid = rel < c.N;
     const uint64_t s = c.first + (valid ? rel : 0);
     // ---- pass 1: both paths, u and 1 / S of every step to the tape ----
@@ -284,26 +284,30 @@ struct SensSpace {
   size_t cap = 0;
   double *h = nullptr;
   size_t h_cap = 0;
-  bool reserve(int dev, size_t bytes, size_t h_doubles) {
+  bool reserve_device(int dev, size_t bytes) {
     if (d && (dev != device || bytes > cap)) release();
     if (!d) {
       if (cudaMalloc(&d, bytes) != cudaSuccess) {
+        (void)cudaGetLastError();
         d = nullptr;
         return false;
       }
       cap = bytes;
       device = dev;
     }
-    if (h_doubles > h_cap) {
-      if (h) cudaFreeHost(h);
+    return true;
+  }
+  bool reserve_host(size_t doubles) {
+    if (doubles <= h_cap) return true;
+    if (h) cudaFreeHost(h);
+    h = nullptr;
+    h_cap = 0;
+    if (cudaHostAlloc((void **)&h, sizeof(double) * doubles, cudaHostAllocDefault) != cudaSuccess) {
+      (void)cudaGetLastError();
       h = nullptr;
-      h_cap = 0;
-      if (cudaHostAlloc((void **)&h, sizeof(double) * h_doubles, cudaHostAllocDefault) != cudaSuccess) {
-        h = nullptr;
-        return false;
-      }
-      h_cap = h_doubles;
+      return false;
     }
+    h_cap = doubles;
     return true;
   }
   void release() {
@@ -357,17 +361,20 @@ extern "C" mlmc_status mlmc_sensitivities(int level, uint64_t N, const mlmc_para
   const size_t tape = sizeof(double) * tape_doubles(c.n, c.m);
   const uint64_t want = std::max<uint64_t>(std::min<uint64_t>((uint64_t)4 * ctx_num_sms(), SENS_MAX_TAPE / tape),
                                            (SENS_KEEP - SENS_KEEP / 8) / tape);
-  const int n_ctas = (int)std::min<uint64_t>(want, (N + SENS_THREADS - 1) / SENS_THREADS);
-  const uint64_t per = (uint64_t)n_ctas * SENS_THREADS;
-  const int iters = (int)((N + per - 1) / per);
+  int n_ctas = (int)std::min<uint64_t>(want, (N + SENS_THREADS - 1) / SENS_THREADS);
   const size_t smem = sizeof(double) * (3 * (size_t)slots(c.n) + (c.m > 0 ? 2 * (size_t)slots(c.m) : 0));
   cudaStream_t st = ctx_stream();
   const size_t rows = (size_t)SENS_ROWS * c.ni, n_res = P_COUNT + rows;
   int dev = 0;
   MLMC_CK(cudaGetDevice(&dev));
-  const size_t doubles = (size_t)n_ctas * (P_COUNT + rows) + n_res;
-  const size_t bytes = (size_t)n_ctas * tape + sizeof(double) * doubles;
-  if (!g_sens.reserve(dev, bytes, n_res)) return MLMC_ENOMEM;
+  if (!g_sens.reserve_host(n_res)) return MLMC_ENOMEM;
+  // any number of CTAs gives the statistics: half as many, down to one, where
+  // the device has no room for their tapes
+  while (!g_sens.reserve_device(dev, sizeof(double) * ((size_t)n_ctas * (tape / sizeof(double) + P_COUNT + rows) + n_res))) {
+    if (n_ctas == 1) return MLMC_ENOMEM;
+    n_ctas = (n_ctas + 1) / 2;
+  }
+  const uint64_t per = (uint64_t)n_ctas * SENS_THREADS, iters = (N + per - 1) / per;
   double *d_tape = (double *)g_sens.d, *d_part = d_tape + (size_t)n_ctas * (tape / sizeof(double));
   double *d_ip = d_part + (size_t)n_ctas * P_COUNT, *d_res = d_ip + (size_t)n_ctas * rows;
   mlmc_status rs = MLMC_OK;
