@@ -433,7 +433,8 @@ mlmc_status mlmc_batch_estimate(const mlmc_params *params, const double *eps, in
  * scheme only (MLMC_EINVAL otherwise).  Synchronous.  Device scratch: 2 KB per
  * fine and coarse step and CTA of 128 samples, 1.07 GB at most (level 10, from
  * 43,521 samples); where the device has less room, fewer CTAs, down to one's 3 MB
- * (MLMC_ENOMEM below that).  Up to 128 MB of it stay allocated for the next call. */
+ * (MLMC_ENOMEM below that).  Up to 128 MB of it stay allocated for the next call
+ * and are given back when another allocation of the library needs the room. */
 typedef struct {
   double A[7];
   double B[7];

@@ -33,6 +33,16 @@ namespace mlmc_host {
 Ctx g;
 
 
+cudaError_t device_malloc(void **p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    (void)cudaGetLastError();
+    if (error_model_release() && (e = cudaMalloc(p, bytes)) != cudaSuccess) (void)cudaGetLastError();
+  }
+  if (e != cudaSuccess) *p = nullptr;
+  return e;
+}
+
 mlmc_status ensure_ctx() {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess) return MLMC_ECUDA;
@@ -59,7 +69,7 @@ mlmc_status m1_table(int d, double **dev, const std::vector<double> **host) {
   if (it == g.m1_dev.end()) {
     const int n = 1 << (d - 1);
     double *p = nullptr;
-    MLMC_CK(cudaMalloc(&p, sizeof(double) * n));
+    MLMC_CK(device_malloc(&p, sizeof(double) * n));
     MLMC_CK(launch_m1_table(d, p, g.st));
     std::vector<double> h(n);
     MLMC_CK(cudaMemcpyAsync(h.data(), p, sizeof(double) * n, cudaMemcpyDeviceToHost, g.st));
@@ -271,7 +281,7 @@ mlmc_status m2_perm_device(int d, int n, const uint16_t **out) {
   std::vector<uint16_t> h(1 << d);
   for (int j = 0; j < (1 << d); ++j) h[j] = (uint16_t)t->pi[j];
   uint16_t *p = nullptr;
-  MLMC_CK(cudaMalloc(&p, sizeof(uint16_t) * h.size()));
+  MLMC_CK(device_malloc(&p, sizeof(uint16_t) * h.size()));
   MLMC_CK(cudaMemcpy(p, h.data(), sizeof(uint16_t) * h.size(), cudaMemcpyHostToDevice));
   g.m2_perm[std::make_pair(d, n)] = p;
   *out = p;
@@ -303,7 +313,7 @@ mlmc_status get_table(int method, int d, int rep, int fZ, const void **out, bool
     if (rep == REP_FIXED) {
       std::vector<int32_t> h(2 * n);
       for (int j = 0; j < 2 * n; ++j) h[j] = (int32_t)std::llround(std::ldexp(m2_value(*t, d, j, rep, fZ), fZ));
-      MLMC_CK(cudaMalloc(&p, sizeof(int32_t) * h.size()));
+      MLMC_CK(device_malloc(&p, sizeof(int32_t) * h.size()));
       MLMC_CK(cudaMemcpy(p, h.data(), sizeof(int32_t) * h.size(), cudaMemcpyHostToDevice));
     } else if (rep == REP_FP16 || rep == REP_BF16) {
       std::vector<uint16_t> h(2 * n);
@@ -311,14 +321,14 @@ mlmc_status get_table(int method, int d, int rep, int fZ, const void **out, bool
         const double v = m2_value(*t, d, j, rep, fZ);
         h[j] = rep == REP_FP16 ? half_bits(v) : bf16_bits(v);
       }
-      MLMC_CK(cudaMalloc(&p, sizeof(uint16_t) * h.size()));
+      MLMC_CK(device_malloc(&p, sizeof(uint16_t) * h.size()));
       MLMC_CK(cudaMemcpy(p, h.data(), sizeof(uint16_t) * h.size(), cudaMemcpyHostToDevice));
     } else {
       return MLMC_EINVAL;
     }
   } else if (method == 1 && full_signed) {
     const size_t es = (rep == REP_FP16 || rep == REP_BF16) ? 2 : 4;
-    MLMC_CK(cudaMalloc(&p, es * 2 * n));
+    MLMC_CK(device_malloc(&p, es * 2 * n));
     MLMC_CK(launch_m1_signed(z64, d, rep, fZ, p, g.st));
     MLMC_CK(cudaStreamSynchronize(g.st));
   } else if (method == 1) {
@@ -326,14 +336,14 @@ mlmc_status get_table(int method, int d, int rep, int fZ, const void **out, bool
       p = z64;
     } else {
       const size_t es = (rep == REP_FP16 || rep == REP_BF16) ? 2 : 4;
-      MLMC_CK(cudaMalloc(&p, es * n));
+      MLMC_CK(device_malloc(&p, es * n));
       MLMC_CK(launch_m1_convert(z64, n, rep, fZ, p, g.st));
       MLMC_CK(cudaStreamSynchronize(g.st));
     }
   } else {
     M3Coef c;
     m3_fit(zh->data(), d, c);
-    MLMC_CK(cudaMalloc(&p, sizeof(M3Coef)));
+    MLMC_CK(device_malloc(&p, sizeof(M3Coef)));
     MLMC_CK(cudaMemcpy(p, &c, sizeof(M3Coef), cudaMemcpyHostToDevice));
   }
   g.tables[key] = p;
@@ -388,7 +398,7 @@ mlmc_status mlmc_icdf_table(int method, int d, int rep, int fZ, double *out) {
   if ((s = get_table(method, d, rep, fZ, &tab)) != MLMC_OK) return s;
   const int n = 1 << (d - 1);
   double *dv = nullptr;
-  MLMC_CK(cudaMalloc(&dv, sizeof(double) * n));
+  MLMC_CK(device_malloc(&dv, sizeof(double) * n));
   cudaError_t e = launch_table_values(method, d, rep, fZ, tab, dv, g.st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, dv, sizeof(double) * n, cudaMemcpyDeviceToHost, g.st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(g.st);
@@ -482,8 +492,8 @@ mlmc_status mlmc_philox(const uint32_t *ctr, uint64_t n, uint64_t seed, uint32_t
   RoundKeys rk;
   make_round_keys(seed, rk);
   uint4 *dc = nullptr, *dout = nullptr;
-  if (cudaMalloc(&dc, 16 * n) != cudaSuccess) return MLMC_ENOMEM;
-  if (cudaMalloc(&dout, 16 * n) != cudaSuccess) { cudaFree(dc); return MLMC_ENOMEM; }
+  if (device_malloc(&dc, 16 * n) != cudaSuccess) return MLMC_ENOMEM;
+  if (device_malloc(&dout, 16 * n) != cudaSuccess) { cudaFree(dc); return MLMC_ENOMEM; }
   cudaError_t e = cudaMemcpyAsync(dc, ctr, 16 * n, cudaMemcpyHostToDevice, g.st);
   if (e == cudaSuccess) e = launch_philox(dc, n, rk, dout, g.st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(out, dout, 16 * n, cudaMemcpyDeviceToHost, g.st);

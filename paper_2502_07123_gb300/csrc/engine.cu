@@ -488,7 +488,7 @@ struct Group {
 
 template <class T>
 bool dev_alloc(T **p, size_t n) {
-  return cudaMalloc((void **)p, sizeof(T) * std::max<size_t>(n, 1)) == cudaSuccess;
+  return device_malloc(p, sizeof(T) * std::max<size_t>(n, 1)) == cudaSuccess;
 }
 
 }  // namespace

@@ -73,6 +73,13 @@ mlmc_status ensure_ctx();
 cudaStream_t ctx_stream();
 // The context's SM count.
 int ctx_num_sms();
+// Gives back the error model's kept device workspace (sens.cu); false: there was none.
+bool error_model_release();
+// cudaMalloc that tries once more without that workspace, and leaves no error
+// for the next launch's check when there is no room.
+cudaError_t device_malloc(void **p, size_t bytes);
+template <class T>
+cudaError_t device_malloc(T **p, size_t bytes) { return device_malloc((void **)p, bytes); }
 
 // ---------------------------------------------------------------------------
 // approximate-Normal tables (context.cu)

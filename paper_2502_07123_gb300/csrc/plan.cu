@@ -120,7 +120,7 @@ bool grow(T *&p, size_t &cap, size_t need) {
   p = nullptr;
   cap = 0;
   const size_t n = std::max(need, cap * 2);
-  if (cudaMalloc(&p, sizeof(T) * n) != cudaSuccess) return false;
+  if (device_malloc(&p, sizeof(T) * n) != cudaSuccess) return false;
   cap = n;
   return true;
 }
@@ -395,10 +395,10 @@ mlmc_status plan_create_impl(mlmc_plan **out, const mlmc_work *work, int n_work,
     *out = pl;
     return MLMC_OK;
   }
-  if (cudaMalloc(&pl->d_items, sizeof(ItemDesc) * ni) != cudaSuccess ||
-      cudaMalloc(&pl->d_partials, sizeof(Partial) * std::max<uint32_t>(1, chunk)) != cudaSuccess ||
-      cudaMalloc(&pl->d_out, sizeof(DevSums) * n_work) != cudaSuccess ||
-      cudaMalloc(&pl->d_counters, sizeof(uint32_t) * ni) != cudaSuccess) {
+  if (device_malloc(&pl->d_items, sizeof(ItemDesc) * ni) != cudaSuccess ||
+      device_malloc(&pl->d_partials, sizeof(Partial) * std::max<uint32_t>(1, chunk)) != cudaSuccess ||
+      device_malloc(&pl->d_out, sizeof(DevSums) * n_work) != cudaSuccess ||
+      device_malloc(&pl->d_counters, sizeof(uint32_t) * ni) != cudaSuccess) {
     free_plan_device(pl);
     delete pl;
     return MLMC_ENOMEM;

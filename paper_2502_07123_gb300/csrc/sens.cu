@@ -276,7 +276,8 @@ __global__ void sens_finalize_kernel(const double *part, const double *inst_part
 
 // Device workspace and pinned result staging, kept between calls (under the
 // library lock, each call synchronises): up to SENS_KEEP bytes, more is given
-// back at the end of the call.
+// back at the end of the call, and all of it when another allocation of the
+// library fails (error_model_release).
 constexpr size_t SENS_KEEP = (size_t)128 << 20, SENS_MAX_TAPE = (size_t)1 << 30;
 struct SensSpace {
   int device = -1;
@@ -319,6 +320,12 @@ struct SensSpace {
 SensSpace g_sens;
 
 }  // namespace
+
+bool mlmc_host::error_model_release() {
+  const bool had = g_sens.d != nullptr;
+  g_sens.release();
+  return had;
+}
 
 extern "C" mlmc_status mlmc_sensitivities(int level, uint64_t N, const mlmc_params *p, uint64_t seed,
                                           uint64_t first_sample, mlmc_sensitivity *out, double *inst_out) {

@@ -1,5 +1,6 @@
 """The error model's device workspace where the device has little room: fewer CTAs
-instead of a refusal."""
+instead of a refusal, the kept part given back to the library's other
+allocations, and no error left behind for the call after a refusal."""
 import numpy as np
 import pytest
 
@@ -49,3 +50,23 @@ def test_statistics_with_fewer_ctas(m, leave, level, N, room):
         np.testing.assert_allclose(got[k], want[k], rtol=1e-12, err_msg=k)
     np.testing.assert_array_equal(got["maxabs"], want["maxabs"])
     assert got["mean"] == pytest.approx(want["mean"], rel=1e-9, abs=1e-12)
+
+
+def test_no_error_left_by_a_refusal(m, leave):
+    P = m.make_params(W.params())
+    m.mlmc_level(3, 1000, P, m.FP32_EXACT, 1)
+    leave(64 * MB)
+    with pytest.raises(m.MLMCError) as e:   # several GB of slots
+        m.Engine(max_slots=200_000, max_level=10)
+    assert e.value.status == m.ENOMEM
+    m.mlmc_level(3, 1000, P, m.FP32_EXACT, 1)
+
+
+def test_kept_workspace_is_given_back(m, leave):
+    """117 MB are kept after a level-6 call; an engine that needs them gets them."""
+    P = m.make_params(W.params())
+    m.mlmc_sensitivities(6, 100_001, P, 5)
+    leave(64 * MB)
+    eng = m.Engine(max_slots=3000, max_level=10)
+    assert eng.stats()["slots"] == 3000
+    eng.close()
