@@ -9,7 +9,10 @@ shared uniforms) with 10^4 samples per level.  Inputs (the work list and
 tables) are resident in device memory when the timed region starts; L2 is
 flushed between steps (256 MiB write) outside the per-step events.
 
-Prints one JSON line.  `--impl reference` times the CPU oracle instead (the
+Prints one JSON line on stdout: the step's figures and a summary of the other
+workloads (contract_line); their rows go to stderr before it ("detail: {...}"),
+since with them the line was 33 KB and its head was lost where only the end of
+the output is kept.  `--impl reference` times the CPU oracle instead (the
 reference arm).  Under torchrun each rank simulates a disjoint sample range
 (first_sample offset by rank), the step time is the max over ranks and the
 value is the path-steps of all ranks per second (weak scaling).
@@ -477,10 +480,47 @@ def main():
                 "integer_items_bit_equal": "%d of %d" % (int_equal, sum(1 for r in res if r["exact_int"])),
                 "real_items_max_rel_err_of_sum": max(real_err) if real_err else None}
     if rank == 0:
-        print(json.dumps(out))
+        print("detail: " + json.dumps(out), file=sys.stderr, flush=True)
+        print(json.dumps(contract_line(out)), flush=True)
     plan.close()
     if world > 1:
         dist.destroy_process_group()
+
+
+def contract_line(out):
+    """The output without its long lists: per-level rows, prices and sample counts of
+    every seed, and sweep points become counts, ranges and medians."""
+    def short(x):
+        return float("%.4g" % x) if isinstance(x, float) else x
+
+    def without(d, *drop):
+        return {k: short(v) for k, v in d.items() if k not in drop}
+
+    line = dict(out)
+    if "bitwidth_optimiser" in out:
+        o = out["bitwidth_optimiser"]
+        line["bitwidth_optimiser"] = dict(without(o, "levels", "variables"), levels=len(o["levels"]),
+                                          bounds_hold=sum(1 for r in o["levels"] if r["bound_holds"]))
+    if "nested_step_optimised_widths" in out:
+        line["nested_step_optimised_widths"] = {k: without(v, "var_corrections_euro")
+                                                for k, v in out["nested_step_optimised_widths"].items()}
+    if "time_to_eps" in out:   # seconds and RMS error over eps of each configuration
+        line["time_to_eps"] = {k: [short(v["s_median"]), short(v.get("rms_err_over_eps"))] if isinstance(v, dict) else short(v)
+                               for k, v in out["time_to_eps"].items() if not k.startswith("speedup_")}
+    for key in ("sweep", "sweep_levels"):
+        if key in out:
+            rates = {}
+            for r in out[key]["rows"]:
+                rates.setdefault(r["variant"], []).append(r["path_steps_per_s"])
+            line[key] = {"scheme": out[key]["scheme"], "points": len(out[key]["rows"]),
+                         "path_steps_per_s": {k: [short(min(v)), short(max(v))] for k, v in rates.items()}}
+    for key in ("serving_sample", "serving"):
+        if key in out:
+            line[key] = [without({k: v for k, v in r.items() if not isinstance(v, (list, dict))}, "graph_captures")
+                         for r in out[key]]
+    if "batched" in out:
+        line["batched"] = without({k: v for k, v in out["batched"].items() if not isinstance(v, (list, dict))})
+    return line
 
 
 def _bs_price(o):
