@@ -316,6 +316,14 @@ struct LevelSim {
   // proved that it cannot leave below first.)
   __device__ __forceinline__ bool over() const { return hi > (AS)ff.limT; }
 
+  // Asian sums leave out S_0 (the first step's S, and the first coarse step's): zero is
+  // added there instead of branching round the sum.  As branches they cut the step loop
+  // into blocks whose steps ran one after another: 8,000 level-10 corrections 92 -> 68 us,
+  // Method 2's 108 -> 80; 1.5e7 level-4 ones 568 -> 523.  The binary16 / bfloat16 and
+  // the FP32 exact kernels keep the branch: Method 2's binary16 corrections 70 against
+  // 75 us, 1.5e7 level-4 FP32 samples 343 against 350.
+  static constexpr bool BRANCH_INNER = HALF || (EST == EST_EXACT && XP == XP_F32);
+
   // ---- exact path (FP32 / FP64) ----
   static __device__ __forceinline__ X lower(X a, X b) {
     if constexpr (XP == XP_F64) return min_f64(b, a);
@@ -533,12 +541,12 @@ struct LevelSim {
         z = exact_normal_f32<PHI_OCT>(Je, phi, phil);
         inc = exact_inc(z, c1, X(1));
       }
-      if constexpr (PC == PC_ASIAN) { if (i > 0) accF = accF + S; }
+      if constexpr (PC == PC_ASIAN) { if (!BRANCH_INNER || i > 0) accF = accF + (BRANCH_INNER || i > 0 ? S : X(0)); }
       S = fma(S, inc, S);
       if constexpr (PC == PC_LOOKBACK) minF = lower(minF, S);
       if constexpr (COARSE) {
         if (odd) {
-          if constexpr (PC == PC_ASIAN) { if (i > 1) accC = accC + Sc; }
+          if constexpr (PC == PC_ASIAN) { if (!BRANCH_INNER || i > 1) accC = accC + (BRANCH_INNER || i > 1 ? Sc : X(0)); }
           if (qinc) {
             // c1_c = 2 c1 and (Z + Z')^2 - 2 = (Z^2 - 1) + (Z'^2 - 1) + 2 Z Z': the coarse
             // increment is the sum of the two fine ones (Milstein: + 2 c3 Z Z')
@@ -637,7 +645,7 @@ struct LevelSim {
       // its own from Z~_2k + Z~_2k+1
 #pragma unroll
       for (int l = 0; l < KP; ++l) {
-        if constexpr (PC == PC_ASIAN) { if (i > 0) aaccF[l] += aS[l]; }
+        if constexpr (PC == PC_ASIAN) aaccF[l] += i > 0 ? aS[l] : 0;
         // lazy runs track S after the odd fine steps only (limT); with the parity
         // unknown at compile time, after every step (more is as exact)
         constexpr bool TRACK_FINE = PAR == 1 || (PAR == -1 && COARSE);
@@ -645,7 +653,7 @@ struct LevelSim {
         if constexpr (PC == PC_LOOKBACK) aminF[l] = aS[l] < aminF[l] ? aS[l] : aminF[l];
         if constexpr (COARSE) {
           if (odd) {
-            if constexpr (PC == PC_ASIAN) { if (i > 1) aaccC[l] += aSc[l]; }
+            if constexpr (PC == PC_ASIAN) aaccC[l] += i > 1 ? aSc[l] : 0;
             fx32_coarse<EAGER>(l, azprev[l], x);
             if constexpr (PC == PC_LOOKBACK) aminC[l] = aSc[l] < aminC[l] ? aSc[l] : aminC[l];
           } else {
@@ -659,13 +667,13 @@ struct LevelSim {
         const uint32_t Jl = l == 0 ? J : (J << (d * l));  // this lane's field at the top
         if constexpr (FIXED) {
           const int32_t z = fixed_z(Jl);
-          if constexpr (PC == PC_ASIAN) { if (i > 0) aaccF[l] += aS[l]; }
+          if constexpr (PC == PC_ASIAN) aaccF[l] += i > 0 ? aS[l] : 0;
           if constexpr (FAST) aS[l] = ff_step<EAGER>(aS[l], z, ff.con1r, ff.mfine, satb[l]);
           else aS[l] = fx_step(aS[l], z, fx.con1A, 1, sat[l]);
           if constexpr (PC == PC_LOOKBACK) aminF[l] = aS[l] < aminF[l] ? aS[l] : aminF[l];
           if constexpr (COARSE) {
             if (odd) {
-              if constexpr (PC == PC_ASIAN) { if (i > 1) aaccC[l] += aSc[l]; }
+              if constexpr (PC == PC_ASIAN) aaccC[l] += i > 1 ? aSc[l] : 0;
               if constexpr (FAST) aSc[l] = ff_step<EAGER>(aSc[l], azprev[l] + z, ff.con1cr, ff.mcoarse, satb[l]);
               else aSc[l] = fx_step(aSc[l], azprev[l] + z, fx.con1cA, 2, sat[l]);
               if constexpr (PC == PC_LOOKBACK) aminC[l] = aSc[l] < aminC[l] ? aSc[l] : aminC[l];
@@ -1120,7 +1128,9 @@ __device__ __forceinline__ void run_group(Sim &sim, Acc &acc, const LaunchArgs &
     const PhiloxStream ps((uint32_t)(qbase >> 32), it.ctr2, it.ctr3, args.rk);
     for (uint32_t c = 0; c < calls; ++c) {
       const uint4 w = Sim::STREAM ? ps.call((uint32_t)qbase + c, args.rk) : draw(it, args, qbase + c);
-      const int i0 = (int)(c << 2);
+      // (a step asks of its index whether it is the first; the binary16 / bfloat16
+      // kernels were faster with the index itself)
+      const int i0 = Sim::HALF ? (int)(c << 2) : c ? 4 : 0;
       sim.template step<true, 0, E>(w.x << lsh, i0);
       sim.template step<true, 1, E>(w.y << lsh, i0 + 1);
       sim.template step<true, 0, E>(w.z << lsh, i0 + 2);
