@@ -54,7 +54,9 @@ constexpr int MAX_THREADS = 256;
 // registers, measured 8-16% faster than their natural ~144), as do the
 // corrections whose natural allocation lies just above.
 // The FP32 exact kernels need 80-96 registers and are held to 80 but for three
-// device-scheduled ones; the binary16 / bfloat16 corrections' static launches
+// device-scheduled ones and the Asian ones, which take 5 CTAs (8,000 level-10
+// samples 56 -> 53 us, 1.2e8 level-1 ones 459 -> 457); the binary16 / bfloat16
+// corrections' static launches
 // need up to 104 and are held to 96, and the unpacked binary16 / bfloat16
 // approximate kernels' (two samples per thread from level 2), 84-96, to 80.
 // Every other instantiation keeps its natural allocation (a cap there spills).
@@ -65,7 +67,7 @@ template <int EST, int XP, int AP, int SCHEME, int PC, int KP, bool DYN = false>
   static constexpr int value =
       EM_TERMINAL_FX32 && EST == EST_APPROX ? 7
       : EM_TERMINAL_FX32 && EST == EST_CORR && !DYN ? 6
-      : EST == EST_EXACT && XP == XP_F32 ? (!DYN || (SCHEME == 0 && PC != PC_ASIAN) ? 6 : 1)
+      : EST == EST_EXACT && XP == XP_F32 ? (!DYN && PC == PC_ASIAN ? 5 : !DYN || (SCHEME == 0 && PC != PC_ASIAN) ? 6 : 1)
       : EST == EST_CORR && FX ? 4
       : EST == EST_CORR && AP != AP_FIXED && !DYN ? (SCHEME == 1 && PC == PC_ASIAN ? 4 : 5)
       : EST == EST_APPROX && AP == AP_FX32 && PC == PC_ASIAN ? 4
