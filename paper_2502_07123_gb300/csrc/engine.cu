@@ -708,14 +708,14 @@ mlmc_status capture(mlmc_engine *e) {
 mlmc_status group_of(mlmc_engine *e, const BuiltItem &b, int threads, uint64_t seed, int *gi) {
   for (int i = 0; i < (int)e->groups.size(); ++i) {
     const Group &G = e->groups[i];
-    if (G.family == b.family && G.scheme == b.scheme && G.pc == b.pc && G.threads == threads && G.smem == b.smem &&
-        G.seed == seed) {
+    if (G.family == b.family && G.scheme == b.scheme && G.pc == b.pc && G.threads == threads &&
+        G.smem == b.smem_class && G.seed == seed) {
       *gi = i;
       return MLMC_OK;
     }
   }
   Group G;
-  G.family = b.family; G.scheme = b.scheme; G.pc = b.pc; G.threads = threads; G.smem = b.smem; G.seed = seed;
+  G.family = b.family; G.scheme = b.scheme; G.pc = b.pc; G.threads = threads; G.smem = b.smem_class; G.seed = seed;
   make_round_keys(seed, G.rk);
   if ((int)e->groups.size() < GMAX) {
     e->groups.push_back(G);

@@ -153,7 +153,8 @@ bool tuning_for(int family, int scheme, int pc, int level, int *threads, int *sp
 struct BuiltItem {
   mlmc::ItemDesc it;
   int family, scheme, pc;
-  size_t smem;
+  size_t smem;          // dynamic shared memory of a static launch (table_form)
+  size_t smem_class;    // the most that items of its family take at its table size (the engine's groups)
   int kp;               // samples per pack
   double cost_step;     // model cost per fine path-step
   double chunk_cost;    // model cost of one chunk (set by chunk_built)

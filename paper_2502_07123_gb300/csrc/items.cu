@@ -394,21 +394,33 @@ int64_t table_zmax_fixed(const double *Z, int d, int method, int fZ, int fields)
   return zmax;
 }
 
-
+int bit_length(uint64_t x) {
+  int n = 0;
+  for (; x; x >>= 1) ++n;
+  return n;
+}
 
 // Level-0 approximate items of the 32-bit fast datapath (families 8 and 15)
 // with a terminal payoff take their sample values from the per-index table
 // (tab_y0), unless they write per-sample records.  Only lazy items: S_0 <=
 // limT there, so no index's one fine step leaves lim_S and no sample counts a
 // saturation (the items that may saturate keep the clamped step code).
-int bit_length(uint64_t x) {
-  int n = 0;
-  for (; x; x >>= 1) ++n;
-  return n;
-}
 int tab_y0_of(const BuiltItem &b, const void *dump) {
   return (b.family == 8 || b.family == 15) && b.it.level == 0 && b.pc == PC_TERMINAL && b.it.ff.lazy && !dump ? 1
                                                                                                               : 0;
+}
+
+// The form of an item's shared-memory table and its size.  The 32-bit datapath's
+// holds an entry per index for every method (Method 3's lines are evaluated into
+// it): 8 bytes (Z~_j, fine sum1_j), with Method 2's ranks behind them, or 4, the
+// level-0 values and the pre-scaled Euler form's P_j (fx32_pre).  At d = 12 the
+// CTAs of a merged launch fit 4 times on an SM with 8 bytes and 6 times with 4.
+void table_form(BuiltItem &b, const void *dump) {
+  const ItemDesc &it = b.it;
+  b.it.tab_y0 = tab_y0_of(b, dump);
+  const bool fx32 = b.family == 8 || b.family == 10 || b.family == 15;
+  const bool four = it.tab_y0 || (it.ff.pre_ok && !dump && b.scheme == MLMC_EULER);
+  b.smem = fx32 && four ? (size_t)4 << it.d : b.smem_class;
 }
 
 // Split an item's sample groups into chunks of `threads` x groups_per_thread.
@@ -637,14 +649,12 @@ mlmc_status build_item(const mlmc_work &w, int out_index, void *dump, BuiltItem 
       default: return MLMC_EINVAL;
     }
   }
-  if (b.family == 8 || b.family == 10 || b.family == 15) {
-    // the 32-bit datapath's shared-memory table: (Z~_j, fine sum1_j) pairs for
-    // every method (Method 3's lines are evaluated into it), then Method 2's ranks
-    b.smem = ((size_t)8 << p->icdf_bits) + (it.perm ? (sizeof(uint16_t) << p->icdf_bits) : 0);
-  }
   b.scheme = p->scheme;
   b.pc = p->payoff == MLMC_ASIAN ? PC_ASIAN : (p->payoff == MLMC_LOOKBACK ? PC_LOOKBACK : PC_TERMINAL);
-  it.tab_y0 = tab_y0_of(b, dump);
+  b.smem_class = b.smem;
+  if (b.family == 8 || b.family == 10 || b.family == 15)
+    b.smem_class = ((size_t)8 << p->icdf_bits) + (it.perm ? (sizeof(uint16_t) << p->icdf_bits) : 0);
+  table_form(b, dump);
   // |Y| <= max(lim_S, 2^f_S) < 2^ybits
   const int ybits = std::max(bit_length((uint64_t)it.ff.limS), it.fx.fS + 1);
   it.y0_bits = std::max(0, 64 - 2 * ybits);
@@ -692,7 +702,7 @@ mlmc_status build_item_cached(const mlmc_work &w, int out_index, void *dump, Bui
   it.N = w.N;
   it.out_index = (uint32_t)out_index;
   it.dump = dump;
-  it.tab_y0 = tab_y0_of(b, dump);
+  table_form(b, dump);
   const uint64_t spc = samples_per_group(lev, b.kp);
   it.g0 = w.first_sample / spc;
   it.g1 = w.N == 0 ? it.g0 : (w.first_sample + w.N + spc - 1) / spc;
