@@ -1686,6 +1686,23 @@ cudaError_t launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t st, cons
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
+  // An approximate kernel's few KB would have its SMs configured for little shared
+  // memory, and a correction kernel beside it (19-25 KB a CTA) then waits for whole SMs
+  // to drain before they can be configured again.  132 KB hold 7 of its CTAs and two of
+  // the other's: an adaptive estimate with enumerated levels 48 -> 39 us.  (All of the
+  // 228 KB on every kernel cost small work lists 2 us; 100 KB did for binary16 only.)
+  // Tables above 16 KB keep the default.
+  if constexpr (EST == EST_APPROX) {
+    static int carved = cudaSharedmemCarveoutDefault, carved_on = -1;
+    const int want = smem <= 16 * 1024 ? 58 : (int)cudaSharedmemCarveoutDefault;   // percent of 228 KB
+    int dev = 0;
+    if (!a.dyn && !occ && !a.dump && cudaGetDevice(&dev) == cudaSuccess && (want != carved || dev != carved_on)) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, want);
+      if (e != cudaSuccess) return e;
+      carved = want;
+      carved_on = dev;
+    }
+  }
   if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, k, (int)block.x, smem);
   k<<<grid, block, smem, st>>>(a);
   return cudaGetLastError();
