@@ -108,4 +108,20 @@ __device__ __forceinline__ bool above_f64(double a, double b) {
   return x > __double_as_longlong(b) && x <= 0x7FF0000000000000LL;
 }
 
+// 1 / x: the hardware's single-precision reciprocal r of x and one cubic step of
+// Newton's iteration, r (1 + e + e^2) with e = 1 - x r (|e| < 2^-21, so what is
+// left out is below 2^-63); by division outside the float range.
+__device__ __forceinline__ double reciprocal(double x) {
+  const int hi = __double2hiint(x), lo = __double2loint(x);
+  const uint32_t mag = (uint32_t)hi & 0x7FFFFFFFu;
+  if (mag - 0x39B00000u >= 0x0C800000u) return 1.0 / x;   // |x| outside [2^-100, 2^100)
+  const float f = __uint_as_float(((mag - 0x38000000u) << 3) | ((uint32_t)lo >> 29));
+  float rf;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rf) : "f"(f));
+  const uint32_t b = __float_as_uint(rf);
+  const double r = __hiloint2double((int)(((b >> 3) + 0x38000000u) | ((uint32_t)hi & 0x80000000u)), (int)(b << 29));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 }  // namespace mlmc
