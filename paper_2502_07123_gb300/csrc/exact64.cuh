@@ -11,7 +11,10 @@
 // path-step, bound by issue and the ALU pipe (53%) with the FP64 unit at 42%.
 // 500,003 level-5 Milstein European samples: 2.25 -> 0.110 ms.  Absolute error of Phi^-1 at most
 // 2^-54, root mean square 2^-57.8 (a correctly rounded FP64 value of [1, 2) is
-// up to 2^-53 off); of the increment 2^-60.
+// up to 2^-53 off).  An increment adds to c2 2^-54 and c3 |Z| 2^-53 of that at most
+// 5 units 2^-qF (Euler: a product up to 4.4 low, the complement's one, q1's half; 10
+// on the coarse path; Milstein 12 and 38; emulated over 3e5 draws 3.3, 5.7, 4.6 and
+// 12.3).  qF is 58 for increments near 8 and 68 below 2^-7 (exact64_consts).
 #pragma once
 #include <stdint.h>
 
@@ -95,7 +98,9 @@ __device__ __forceinline__ double q_to_double(int64_t v, uint32_t hi0) {
 }
 
 // min(x, y) of doubles by integer comparison (the FP64 comparison runs at the
-// FP64 rate); a NaN from arithmetic (positive sign) loses, as in fmin.
+// FP64 rate).  A NaN of positive sign loses, one of negative sign wins; the path
+// minimum may be either, since the payoff subtracts it from a terminal value that
+// is NaN from the same step on.
 __device__ __forceinline__ double min_f64(double x, double y) {
   const int64_t a = __double_as_longlong(x), b = __double_as_longlong(y);
   const int64_t ka = a ^ (int64_t)((uint64_t)(a >> 63) >> 1), kb = b ^ (int64_t)((uint64_t)(b >> 63) >> 1);

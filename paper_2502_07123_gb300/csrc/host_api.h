@@ -144,8 +144,8 @@ extern std::map<std::tuple<int, int, int, int>, std::pair<int, int>> g_tune;
 // Incremented on every change of g_tune (keys of the plan cache).
 extern uint64_t g_tune_gen;
 int level_class(int level);
-// Launch shape (CTA threads, fine path-steps per thread) of a kernel class.
-// Launch shape of a kernel class; true: the default one (chunk_count's grow).
+// Launch shape (CTA threads, fine path-steps per thread) of a kernel class; true:
+// the default one (chunk_count's grow).
 bool tuning_for(int family, int scheme, int pc, int level, int *threads, int *spt);
 
 // A work item with its constants and tables resolved (build_item), before

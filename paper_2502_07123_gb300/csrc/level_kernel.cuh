@@ -1542,7 +1542,7 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
       uint16_t *pd = (uint16_t *)(smem_tab + (size_t)n * TabBytes<AP>::value);
       for (int k = threadIdx.x; k < n; k += blockDim.x) pd[k] = it.perm[k];
     }
-    // merged launch: only the correction chunks (kind 2) run the FP32 exact path
+    // (the cubics, where this chunk staged them)
     copies_done();
     __syncthreads();
   } else if constexpr (AP != AP_NONE) {
