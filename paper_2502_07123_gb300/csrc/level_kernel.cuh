@@ -1470,7 +1470,9 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
     }
     if (lane == 0) s_item = lo;
   }
-  copies_done();   // of the exact path's table, started before the first chunk
+  // the exact path's table, started before the first chunk: a static launch with an
+  // approximate table waits for it at the barrier behind that table's stores
+  if (AP == AP_NONE || staged) copies_done();
   __syncthreads();
   const int item = s_item;
   const ItemDesc &it = items[item];
@@ -1542,7 +1544,6 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
       uint16_t *pd = (uint16_t *)(smem_tab + (size_t)n * TabBytes<AP>::value);
       for (int k = threadIdx.x; k < n; k += blockDim.x) pd[k] = it.perm[k];
     }
-    // (the cubics, where this chunk staged them)
     copies_done();
     __syncthreads();
   } else if constexpr (AP != AP_NONE) {
@@ -1566,6 +1567,7 @@ __device__ __forceinline__ int stage_chunk(const ItemDesc *items, int n_items, u
         for (int k = threadIdx.x; k < (int)(sizeof(M3Coef) / 4); k += blockDim.x)
           ((uint32_t *)smem_tab)[k] = src[k];
       }
+      copies_done();
       __syncthreads();
     }
   }
