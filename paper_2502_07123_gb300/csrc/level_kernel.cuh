@@ -1688,15 +1688,17 @@ cudaError_t launch_one(dim3 grid, dim3 block, size_t smem, cudaStream_t st, cons
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  // An approximate kernel's few KB would have its SMs configured for little shared
-  // memory, and a correction kernel beside it (19-25 KB a CTA) then waits for whole SMs
-  // to drain before they can be configured again.  132 KB hold 7 of its CTAs and two of
-  // the other's: an adaptive estimate with enumerated levels 48 -> 39 us.  (All of the
-  // 228 KB on every kernel cost small work lists 2 us; 100 KB did for binary16 only.)
-  // Tables above 16 KB keep the default.
+  // An approximate kernel alone runs with the shared memory that its own CTAs take, and
+  // an enumerating one held up the correction kernel beside it (19-25 KB a CTA) until
+  // its SMs were free.  With room for both, 132 KB for fixed point and 100 KB for the
+  // 2-byte tables, an adaptive estimate with enumerated levels takes 49 -> 41 and 41 ->
+  // 34 us.  (100 KB did nothing for fixed point; 132 KB cost 1e6 level-8 binary16 samples
+  // 1.1 us, all 228 KB 4; 64 KB took residency from the deep bfloat16 items.)  Tables
+  // above 16 KB keep the default.
   if constexpr (EST == EST_APPROX) {
     static int carved = cudaSharedmemCarveoutDefault, carved_on = -1;
-    const int want = smem <= 16 * 1024 ? 58 : (int)cudaSharedmemCarveoutDefault;   // percent of 228 KB
+    constexpr bool INT_TABLE = AP == AP_FIXED || AP == AP_FX32 || AP == AP_FX64;
+    const int want = smem > 16 * 1024 ? (int)cudaSharedmemCarveoutDefault : INT_TABLE ? 58 : 44;   // percent of 228 KB
     int dev = 0;
     if (!a.dyn && !occ && !a.dump && cudaGetDevice(&dev) == cudaSuccess && (want != carved || dev != carved_on)) {
       const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, want);
